@@ -1,0 +1,200 @@
+// FP32 D2Q4 steps at omega = 1 on the moments (lbrs_march.cuh): the launchers and the kernels
+// that lead from stored distributions into the moments and back.
+#include <math.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include "lbrs_march.cuh"
+#include "lbrs_launch.h"
+
+namespace lbrs {
+
+namespace {
+
+constexpr int kSMs = 152, kWarpsPerSM = 16;   // the march's registers allow 16 one-warp blocks per SM
+
+// Moments of the next step's pull from stored distributions: U = sum_q f*_q(x - c_q).
+__global__ void __launch_bounds__(256) pull_moments_2d_kernel(const StepArgs<float> a, float* __restrict__ U)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= a.nx || j >= a.ny) return;
+    const int64_t c = (int64_t)j * a.nx + i;
+    float f[4][4];
+    if (i > 0 && i < a.nx - 1 && j > 0 && j < a.ny - 1) {
+        const int64_t s[4] = {c + a.nx + 1, c + a.nx - 1, c - a.nx - 1, c - a.nx + 1};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) f[q][k] = a.src[LBRS_IX((q * 4 + k) * a.N + s[q], 16 * a.N, 50)];
+    } else {
+        pull_edge_2d<float, false>(a, i, j, f);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        U[LBRS_IX(k * a.N + c, 4 * a.N, 50)] =
+            __fadd_rn(__fadd_rn(__fadd_rn(f[0][k], f[1][k]), f[2][k]), f[3][k]);
+}
+
+// f* = f^eq(U) into the populations' planes, two cells a thread.
+__global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restrict__ U, float* __restrict__ f, int64_t N,
+                                                            float c, float gm1)
+{
+    const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= N) return;
+    const bool two = i + 1 < N, vec = (N & 1) == 0;      // vec: every plane starts on 8 bytes
+    MarchConst m;
+    m.c = pk(c, c);
+    m.nc = pk(-c, -c);
+    m.gm1 = pk(gm1, gm1);
+    m.ngm1 = pk(-gm1, -gm1);
+    m.half = pk(0.5f, 0.5f);
+    m.quarter = pk(0.25f, 0.25f);
+    m.one = pk(1.f, 1.f);
+    P2 u[4], e[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float* p = U + k * N + i;
+        u[k] = vec ? *reinterpret_cast<const P2*>(p) : pk(p[0], two ? p[1] : p[0]);
+    }
+    const MarchPrim pr = march_prim(u[0], u[1], u[2], u[3], m);
+    auto store = [&](int k) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float* p = f + (q * 4 + k) * N + i;
+            if (vec) {
+                *reinterpret_cast<P2*>(p) = e[q];
+            } else {
+                p[0] = lo2(e[q]);
+                if (two) p[1] = hi2(e[q]);
+            }
+        }
+    };
+    march_feq<0>(u, pr, m, e);
+    store(0);
+    march_feq<1>(u, pr, m, e);
+    store(1);
+    march_feq<2>(u, pr, m, e);
+    store(2);
+    march_feq<3>(u, pr, m, e);
+    store(3);
+}
+
+// Rows a warp stores.  Fewer rows mean more warps to hide latencies, and more rows recomputed
+// around each warp's own (2 K of them).  An iteration (K source rows) takes 0.33 us by itself and
+// 0.17 us of an SM sub-partition's issue slots (K = 2, measured on 1024^2 and 4096 x 1024), so with w
+// warps on the fullest sub-partition a launch takes about (rows + 2 K) max(0.33, 0.17 w) us; the rule
+// takes the minimum over the rows (1024^2: 16 rows 10.1 us, 8 rows 11.0, 30 rows 15.3; 4096 x 1024:
+// 30 rows 29.3, 12 rows 31.8).  The warps beside y sides that are not periodic take longer per row
+// (0.40 us by themselves, 0.60 beside a wall) and get as many rows as keep them from ending last.
+void march_rows_for(MarchArgs& a, int own, int steps)
+{
+    a.strips = (a.nx + own - 1) / own;
+    const bool per = a.bc[2] == BC_PERIODIC;
+    const double lone = a.bc[2] == BC_WALL || a.bc[3] == BC_WALL ? 0.60 : 0.40;
+    double best = 0.0;
+    for (int rows = 4; rows <= 64; rows += 2) {
+        int end = 0;
+        int64_t chunks = (a.ny + rows - 1) / rows;
+        const int64_t per_sm = (a.strips * chunks + kSMs - 1) / kSMs;
+        const double sub = per_sm <= kWarpsPerSM ? (double)((per_sm + 3) / 4) : (double)per_sm / 4.0 + 0.5;
+        const double resident = fmin(sub, kWarpsPerSM / 4);
+        double t = (rows + 2 * steps) * fmax(0.33, 0.17 * sub);
+        if (!per) {
+            const double iteration = lone + 0.17 * (resident - 1.0);     // beside a y side
+            end = (int)((rows + 2 * steps) * fmax(0.33, 0.17 * resident) / iteration) - steps;
+            end = end < 2 ? 2 : (end > rows ? rows : end);
+            if (a.ny > 2 * end) {
+                chunks = 2 + (a.ny - 2 * end + rows - 1) / rows;
+            } else {
+                end = 0;
+                t = fmax(t, (rows + steps) * iteration);
+            }
+        }
+        if (best == 0.0 || t < best) {
+            best = t;
+            a.rows = rows;
+            a.end_rows = end;
+            a.chunks = (int)chunks;
+        }
+    }
+}
+
+template <int K, bool RECORD>
+cudaError_t launch_k(MarchArgs a, cudaStream_t s)
+{
+    march_rows_for(a, MarchShape<K>::own, K);
+    const int64_t blocks = (int64_t)a.strips * a.chunks;
+    if (a.nx & 1) march2d_kernel<K, true, RECORD><<<(unsigned)blocks, 32, 0, s>>>(a);
+    else march2d_kernel<K, false, RECORD><<<(unsigned)blocks, 32, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool march_enabled()
+{
+    static const int v = [] {
+        const char* e = getenv("LBRS_F32_MARCH");
+        return (e && !strcmp(e, "0")) ? 0 : 1;
+    }();
+    return v != 0;
+}
+
+// f^eq of the Dirichlet sides' states in FP64, rounded: the values of the device's ghost table
+// (the same operations in the same order; no contraction on either side).
+void march_ghosts(const GhostSpec& g, double gamma, double c, float out[4][16])
+{
+    for (int s = 0; s < 4; ++s) {
+        for (int n = 0; n < 16; ++n) out[s][n] = 0.f;
+        if (g.kind[s] != BC_DIRICHLET) continue;
+        const double rho = g.prim[s][0], u0 = g.prim[s][1], v0 = g.prim[s][2], p0 = g.prim[s][3];
+        const double U[4] = {rho, rho * u0, rho * v0, p0 / (gamma - 1.0) + 0.5 * rho * (u0 * u0 + v0 * v0)};
+        const double u = U[1] / U[0], v = U[2] / U[0];
+        const double p = (gamma - 1.0) * (U[3] - 0.5 * (U[1] * u + U[2] * v));
+        const double F[4] = {U[1], U[1] * u + p, U[1] * v, u * (U[3] + p)};
+        const double G[4] = {U[2], U[2] * u, U[2] * v + p, v * (U[3] + p)};
+        for (int k = 0; k < 4; ++k) {
+            const double a = 0.25 * U[k], b = c * F[k], d = c * G[k];
+            out[s][k] = (float)((a - b) - d);
+            out[s][4 + k] = (float)((a + b) - d);
+            out[s][8 + k] = (float)((a + b) + d);
+            out[s][12 + k] = (float)((a - b) + d);
+        }
+    }
+}
+
+cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaStream_t s)
+{
+    MarchArgs a;
+    a.src = st.src;
+    a.dst = st.dst;
+    memcpy(a.ghost, st.ghost, sizeof a.ghost);
+    a.N = st.N;
+    a.nx = st.nx;
+    a.ny = st.ny;
+    for (int n = 0; n < 4; ++n) a.bc[n] = st.bc[n];
+    a.c = st.c;
+    a.gm1 = st.gm1;
+    if (record) return steps == 2 ? launch_k<2, true>(a, s) : launch_k<1, true>(a, s);
+    return steps == 2 ? launch_k<2, false>(a, s) : launch_k<1, false>(a, s);
+}
+
+cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s)
+{
+    const dim3 block(64, 4);
+    const dim3 grid((unsigned)((a.nx + 63) / 64), (unsigned)((a.ny + 3) / 4));
+    pull_moments_2d_kernel<<<grid, block, 0, s>>>(a, U);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s)
+{
+    const int64_t threads = (N + 1) / 2;
+    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, N, c, gm1);
+    return cudaGetLastError();
+}
+
+LBRS_DEBUG_WORD(debug_word_march)
+
+}  // namespace lbrs

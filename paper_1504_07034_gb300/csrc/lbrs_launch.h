@@ -36,6 +36,7 @@ struct BatchTile;
 unsigned long long debug_word_f32(int clear);
 unsigned long long debug_word_f64(int clear);
 unsigned long long debug_word_f16(int clear);
+unsigned long long debug_word_march(int clear);
 
 // Failure-detection self-test: a bounded wait on an mbarrier that nothing completes
 // gives up and raises *wait_flag (one block, 4096 polls).
@@ -144,6 +145,27 @@ cudaError_t launch_adjoint_seed(int Q, int K, int storage_f64, const void* dLdU,
 cudaError_t launch_density_loss(int Q, int K, int storage_f64, const void* fs, const void* target, int t_dtype,
                                 void* gbar, int64_t N, int64_t plane, double cell_volume, double* partials, double* out,
                                 cudaStream_t s);
+
+// FP32 D2Q4 at omega = 1 on the moments (lbrs_march.cuh, lbrs_kernels_march.cu): `steps` (1 or 2)
+// steps U -> U' in one launch, bit-identical to the storing kernels' moments.  With record, dst
+// receives the moments of every step, [steps][4][N].  The y sides may be of any kind but halfway
+// walls; off when the environment sets LBRS_F32_MARCH=0.
+struct MarchStep {
+    const float* src;          // U [4][N]
+    float* dst;                // U [4][N] or [steps][4][N], not src
+    float ghost[4][16];        // f^eq of the Dirichlet sides (march_ghosts)
+    int64_t N;
+    int nx, ny;
+    int bc[4];
+    float c, gm1;
+};
+bool march_enabled();
+
+void march_ghosts(const GhostSpec& g, double gamma, double c, float out[4][16]);
+cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaStream_t s);
+// From stored distributions (a.src) the moments U of the next step, and f* = f^eq(U) back.
+cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s);
+cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s);
 
 // Batched D1Q2 / D1Q3 tubes with temporal blocking (lbrs_batch.cuh): one CTA of
 // `block` threads per active tile; dynamic shared memory 2*3Q*(TILE+2H) elements.

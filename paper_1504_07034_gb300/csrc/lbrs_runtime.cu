@@ -128,6 +128,8 @@ struct lbrs_ctx {
     TileMap tmap3[2];        // the same for the three-step kernel (larger boxes)
     int graph_launches[2];   // kernels in graph[b]
     const uint8_t* solid;    // caller-owned obstacle mask [ny][nx] (lbrs_set_obstacles), or NULL
+    cudaGraphExec_t mgraph[2];   // kGraphSteps steps on the moments held in buffer b
+    float mghost[4][16];     // the march's copy of the ghost table
     GhostSpec gspec;         // the sides' kinds and states (the adaptive run rebuilds the ghosts)
     bool adapt_ready;        // the adaptive record holds the current state's run
     bool adapt_used;         // the distributions carry an adaptive lambda
@@ -137,6 +139,7 @@ struct lbrs_ctx {
     char* adj_ws;
     size_t adj_bytes;
     int64_t adj_n, adj_seg, adj_step0;
+    bool adj_moments;        // its checkpoints after the first hold moments
     char err[512];
 };
 
@@ -373,6 +376,36 @@ bool fused3(const lbrs_ctx* ctx)
     return ctx->tmap3[0].valid && ctx->tmap3[1].valid;
 }
 
+// FP32 at omega = 1 (distributions or moments-only storage) on the moments by the marching kernel
+// (lbrs_march.cuh), two steps a launch?  Not with internal walls (solid cells carry distributions
+// that are no equilibria) or halfway walls; the switches that ask for one, two or three storing
+// steps a launch turn it off as well.
+bool march(const lbrs_ctx* ctx)
+{
+    if (ctx->f64 || ctx->f16 || ctx->lattice != LBRS_D2Q4 || ctx->cfg.omega != 1.0 || ctx->solid) return false;
+    if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
+    return march_enabled() && (ctx->f32u ? step2_f32u_enabled() : step2_f32_enabled() && step3_f32_enabled());
+}
+
+MarchStep march_step(const lbrs_ctx* ctx, const char* src, char* dst)
+{
+    MarchStep m;
+    m.src = (const float*)src;
+    m.dst = (float*)dst;
+    memcpy(m.ghost, ctx->mghost, sizeof m.ghost);
+    m.N = ctx->N;
+    m.nx = (int)ctx->cfg.nx;
+    m.ny = (int)ctx->ny_store;
+    for (int s = 0; s < 4; ++s) m.bc[s] = kernel_bc(ctx, s);
+    m.c = (float)ctx->c;
+    m.gm1 = (float)(ctx->cfg.gamma - 1.0);
+    return m;
+}
+
+// Distribution storage enters and leaves the moments once per call (80 + 80 B per cell, two
+// launches): worth it from this many steps on (1024^2: 6 steps in 52 us instead of 80 us).
+constexpr int64_t kMarchMin = 6;
+
 // Steps the next launch takes out of `left`: three where the three-step kernel applies (but
 // 2 + 2 rather than 3 + 1), else two where the two-step kernel does, else one.
 int next_launch_steps(const lbrs_ctx* ctx, int64_t left)
@@ -407,23 +440,40 @@ int readout_lattice(const lbrs_ctx* ctx)
     return lat_code(ctx->lattice);
 }
 
-// Capture graph_steps() steps starting from buffer `from` into graph[from].
-lbrs_status ensure_graph(lbrs_ctx* ctx, int from)
+// Two places for moments: the state buffers themselves in the moments-only form, halves of the idle
+// buffer in the distribution form (64 B per cell hold two sets of moments).
+void march_buffers(const lbrs_ctx* ctx, char* v[2])
 {
-    if (ctx->graph[from]) return LBRS_OK;
+    if (ctx->f32u) {
+        v[0] = ctx->f[ctx->cur];
+        v[1] = ctx->f[ctx->cur ^ 1];
+    } else {
+        v[0] = ctx->f[ctx->cur ^ 1];
+        v[1] = v[0] + 16 * (size_t)ctx->N;
+    }
+}
+
+// n steps on the moments from v[0]; with whole pairs they end in v[n / 2 % 2].
+cudaError_t launch_march_run(const lbrs_ctx* ctx, char* const v[2], int64_t n, cudaStream_t s, int* launches)
+{
+    int b = 0;
+    for (; n > 0; b ^= 1, ++*launches) {
+        const int m = n >= 2 ? 2 : 1;
+        const cudaError_t e = launch_march_f32(march_step(ctx, v[b], v[b ^ 1]), m, false, s);
+        if (e != cudaSuccess) return e;
+        n -= m;
+    }
+    return cudaSuccess;
+}
+
+// Capture `body` (a function enqueuing launches on a stream) into *exec unless it is there.
+template <class Body>
+lbrs_status ensure_graph_of(lbrs_ctx* ctx, cudaGraphExec_t* exec, Body&& body)
+{
+    if (*exec) return LBRS_OK;
     if (!ctx->cap_stream) LBRS_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
     LBRS_CUDA(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t le = cudaSuccess;
-    int b = from, launches = 0;
-    const int G = graph_steps(ctx);
-    for (int n = 0; n < G && le == cudaSuccess; ++launches) {
-        const int m = next_launch_steps(ctx, G - n);
-        le = m == 3 ? launch_step3(ctx, b, ctx->cap_stream)
-                    : (m == 2 ? launch_step2(ctx, b, ctx->cap_stream) : launch_one_step(ctx, b, ctx->cap_stream));
-        n += m;
-        b ^= 1;
-    }
-    ctx->graph_launches[from] = launches;
+    const cudaError_t le = body(ctx->cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &g);
     if (le != cudaSuccess) {
@@ -431,13 +481,31 @@ lbrs_status ensure_graph(lbrs_ctx* ctx, int from)
         return cuda_fail(ctx, le, "step launch during graph capture");
     }
     if (ee != cudaSuccess) return cuda_fail(ctx, ee, "cudaStreamEndCapture");
-    cudaError_t ie = cudaGraphInstantiate(&ctx->graph[from], g, 0);
+    cudaError_t ie = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) {
-        ctx->graph[from] = nullptr;
+        *exec = nullptr;
         return cuda_fail(ctx, ie, "cudaGraphInstantiate");
     }
     return LBRS_OK;
+}
+
+// Capture graph_steps() steps starting from buffer `from` into graph[from].
+lbrs_status ensure_graph(lbrs_ctx* ctx, int from)
+{
+    return ensure_graph_of(ctx, &ctx->graph[from], [&](cudaStream_t s) {
+        cudaError_t le = cudaSuccess;
+        int b = from, launches = 0;
+        const int G = graph_steps(ctx);
+        for (int n = 0; n < G && le == cudaSuccess; ++launches) {
+            const int m = next_launch_steps(ctx, G - n);
+            le = m == 3 ? launch_step3(ctx, b, s) : (m == 2 ? launch_step2(ctx, b, s) : launch_one_step(ctx, b, s));
+            n += m;
+            b ^= 1;
+        }
+        ctx->graph_launches[from] = launches;
+        return le;
+    });
 }
 
 size_t field_bytes(const lbrs_ctx* ctx, int dtype)
@@ -615,12 +683,50 @@ cudaError_t launch_record_step3(lbrs_ctx* ctx, void* Uout)
     return launch_step3_f32(a, &ctx->tmap3[ctx->cur], wait_flag(ctx), ctx->stream);
 }
 
-// n recording steps from the current buffer into U_hist (stride: one step's moments),
-// in threes where the three-step kernel applies (but 2 + 2 rather than 3 + 1), then in pairs
-// where the two-step kernel does.
+// n steps on the moments from `src`, recorded into U_hist[0 .. n): two a launch.
+lbrs_status record_march(lbrs_ctx* ctx, const char* src, int64_t n, char* U_hist)
+{
+    const size_t stride = 16 * (size_t)ctx->N;
+    for (int64_t m = 0; m < n;) {
+        const int k = n - m >= 2 ? 2 : 1;
+        LBRS_CUDA(ctx, launch_march_f32(march_step(ctx, src, U_hist + m * stride), k, true, ctx->stream));
+        ctx->launches += 1;
+        m += k;
+        src = U_hist + (m - 1) * stride;
+    }
+    return LBRS_OK;
+}
+
+// The moments of the first step from the stored distributions f, into U.
+cudaError_t launch_pull_into(lbrs_ctx* ctx, const char* f, char* U)
+{
+    StepArgs<float> a = step_args<float>(ctx, ctx->cur);
+    a.src = (const float*)f;
+    ctx->launches += 1;
+    return launch_pull_moments_f32(a, (float*)U, ctx->stream);
+}
+
+// The current buffer's distributions from the moments U at omega = 1.
+cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U)
+{
+    ctx->launches += 1;
+    return launch_equilibria_f32((const float*)U, (float*)ctx->f[ctx->cur], ctx->N, (float)ctx->c,
+                                 (float)(ctx->cfg.gamma - 1.0), ctx->stream);
+}
+
+// n recording steps from the current buffer into U_hist (stride: one step's moments): on the
+// moments where the march applies; else in threes where the three-step kernel does (but 2 + 2
+// rather than 3 + 1), then in pairs where the two-step kernel does.
 lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
 {
     const size_t stride = (size_t)ctx->K * ctx->N * elem_bytes(ctx);
+    if (march(ctx) && n >= kMarchMin) {
+        LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], U_hist));
+        lbrs_status st = record_march(ctx, U_hist, n - 1, U_hist + stride);
+        if (st != LBRS_OK) return st;
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, U_hist + (n - 1) * stride));
+        return LBRS_OK;
+    }
     int64_t m = 0;
     for (; m + 3 <= n && n - m != 4 && fused3(ctx); m += 3) {
         LBRS_CUDA(ctx, launch_record_step3(ctx, U_hist + m * stride));
@@ -719,7 +825,7 @@ lbrs_status lbrs_debug_check(uint64_t* first)
 {
     if (!first) return fail(nullptr, LBRS_EINVAL, "first is NULL");
     unsigned long long w = 0ull;
-    for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1)})
+    for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1), debug_word_march(1)})
         if (!w) w = v;
     *first = (uint64_t)w;
     if (w)
@@ -795,6 +901,7 @@ lbrs_status lbrs_create(const lbrs_config* cfg, void* d_workspace, size_t bytes,
         for (int k = 0; k < 4; ++k) g.prim[s][k] = cfg->bc[s].prim[k];
     }
     ctx->gspec = g;
+    if (cfg->lattice == LBRS_D2Q4) march_ghosts(g, cfg->gamma, ctx->c, ctx->mghost);
     const int lat = lat_code(cfg->lattice);
     cudaError_t e = launch_ghost(lat, ctx->f64, g, cfg->gamma, ctx->c, ctx->ws + L.ghost, ctx->stream);
     if (e != cudaSuccess) {
@@ -824,6 +931,7 @@ void lbrs_destroy(lbrs_ctx* ctx)
     for (int b = 0; b < 2; ++b) {
         if (ctx->graph[b]) cudaGraphExecDestroy(ctx->graph[b]);
         if (ctx->agraph[b]) cudaGraphExecDestroy(ctx->agraph[b]);
+        if (ctx->mgraph[b]) cudaGraphExecDestroy(ctx->mgraph[b]);
     }
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     free(ctx);
@@ -895,6 +1003,46 @@ lbrs_status lbrs_step(lbrs_ctx* ctx, int64_t n)
     return LBRS_OK;
 }
 
+// n steps at omega = 1 on the moments.  Distribution storage enters through the pull of the first
+// step and leaves through the equilibria of the last, back into the buffer it came from.
+static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
+{
+    char* v[2];
+    march_buffers(ctx, v);
+    const int buf = ctx->f32u ? ctx->cur : ctx->cur ^ 1;
+    int64_t left = n;
+    int launches = 0;
+    if (!ctx->f32u) {
+        LBRS_CUDA(ctx, launch_pull_moments_f32(step_args<float>(ctx, ctx->cur), (float*)v[0], ctx->stream));
+        left -= 1;
+        launches += 1;
+    }
+    if (graphs && left >= 2 * kGraphSteps) {
+        lbrs_status st = ensure_graph_of(ctx, &ctx->mgraph[buf], [&](cudaStream_t s) {
+            int dummy = 0;
+            return launch_march_run(ctx, v, kGraphSteps, s, &dummy);   // an even number of launches: back in v[0]
+        });
+        if (st != LBRS_OK) return st;
+        for (; left >= kGraphSteps; left -= kGraphSteps) {
+            LBRS_CUDA(ctx, cudaGraphLaunch(ctx->mgraph[buf], ctx->stream));
+            launches += kGraphSteps / 2;
+        }
+    }
+    int rest = 0;
+    LBRS_CUDA(ctx, launch_march_run(ctx, v, left, ctx->stream, &rest));
+    launches += rest;
+    if (ctx->f32u) {
+        ctx->cur ^= rest & 1;
+    } else {
+        LBRS_CUDA(ctx, launch_equilibria_f32((const float*)v[rest & 1], (float*)ctx->f[ctx->cur], ctx->N, (float)ctx->c,
+                                             (float)(ctx->cfg.gamma - 1.0), ctx->stream));
+        launches += 1;
+    }
+    ctx->step += n;
+    ctx->launches += launches;
+    return LBRS_OK;
+}
+
 static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
 {
     if (blocked_1d(ctx)) {
@@ -910,6 +1058,7 @@ static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
     }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBRS_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
+    if (march(ctx) && (ctx->f32u || n >= kMarchMin)) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
     int64_t left = n;
     const int G = graph_steps(ctx);
     if (cap == cudaStreamCaptureStatusNone && n >= 2 * G) {
@@ -1541,15 +1690,45 @@ lbrs_status lbrs_forward_checkpointed(lbrs_ctx* ctx, int64_t n_steps, int64_t se
     char* ws = (char*)d_adj_ws;
     ctx->adj_ws = nullptr;
     ctx->adj_step0 = ctx->step;
-    for (int64_t s = 0; s < A.nseg; ++s) {
-        LBRS_CUDA(ctx, cudaMemcpyAsync(ws + A.ckpt0 + s * A.ckpt_stride, ctx->f[ctx->cur], ctx->L.f_bytes,
+    // at omega = 1 the run stays on the moments from its first step on: a checkpoint after the first
+    // holds them (16 instead of 64 B per cell), written by the launch that ends its segment
+    ctx->adj_moments = march(ctx) && ctx->cfg.diag_every <= 0;
+    if (ctx->adj_moments) {
+        char* v[2];
+        march_buffers(ctx, v);
+        LBRS_CUDA(ctx, cudaMemcpyAsync(ws + A.ckpt0, ctx->f[ctx->cur], ctx->L.f_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+        const char* at = nullptr;            // the moments after `done` steps
+        for (int64_t s = 0, done = 0; s < A.nseg; ++s) {
+            const int64_t end = (s + 1) * segment <= n_steps ? (s + 1) * segment : n_steps;
+            char* ckpt = ws + A.ckpt0 + (s + 1) * A.ckpt_stride;
+            int b = 0;
+            while (done < end) {
+                const int m = done == 0 || end - done == 1 ? 1 : 2;
+                char* to = done + m == end ? ckpt : v[b];
+                if (done == 0) {
+                    LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], to));
+                } else {
+                    LBRS_CUDA(ctx, launch_march_f32(march_step(ctx, at, to), m, false, ctx->stream));
+                    ctx->launches += 1;
+                }
+                at = to;
+                b ^= 1;
+                done += m;
+            }
+        }
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, at));
+        ctx->step += n_steps;
+    } else {
+        for (int64_t s = 0; s < A.nseg; ++s) {
+            LBRS_CUDA(ctx, cudaMemcpyAsync(ws + A.ckpt0 + s * A.ckpt_stride, ctx->f[ctx->cur], ctx->L.f_bytes,
+                                           cudaMemcpyDeviceToDevice, ctx->stream));
+            const int64_t len = (s + 1) * segment <= n_steps ? segment : n_steps - s * segment;
+            st = lbrs_step(ctx, len);
+            if (st != LBRS_OK) return st;
+        }
+        LBRS_CUDA(ctx, cudaMemcpyAsync(ws + A.ckpt0 + A.nseg * A.ckpt_stride, ctx->f[ctx->cur], ctx->L.f_bytes,
                                        cudaMemcpyDeviceToDevice, ctx->stream));
-        const int64_t len = (s + 1) * segment <= n_steps ? segment : n_steps - s * segment;
-        st = lbrs_step(ctx, len);
-        if (st != LBRS_OK) return st;
     }
-    LBRS_CUDA(ctx, cudaMemcpyAsync(ws + A.ckpt0 + A.nseg * A.ckpt_stride, ctx->f[ctx->cur], ctx->L.f_bytes,
-                                   cudaMemcpyDeviceToDevice, ctx->stream));
     ctx->adj_ws = ws;
     ctx->adj_bytes = bytes;
     ctx->adj_n = n_steps;
@@ -1579,9 +1758,17 @@ lbrs_status lbrs_backward_checkpointed(lbrs_ctx* ctx, void* d_adj_ws, const void
         const int64_t start = s * ctx->adj_seg;
         const int64_t len = start + ctx->adj_seg <= ctx->adj_n ? ctx->adj_seg : ctx->adj_n - start;
         // recompute the segment from its checkpoint, recording U^{start+1 .. start+len}
-        LBRS_CUDA(ctx, cudaMemcpyAsync(ctx->f[ctx->cur], ws + A.ckpt0 + s * A.ckpt_stride, ctx->L.f_bytes,
-                                       cudaMemcpyDeviceToDevice, ctx->stream));
-        lbrs_status rs = record_steps(ctx, len, uhist);
+        const char* ckpt = ws + A.ckpt0 + s * A.ckpt_stride;
+        lbrs_status rs;
+        if (!ctx->adj_moments) {
+            LBRS_CUDA(ctx, cudaMemcpyAsync(ctx->f[ctx->cur], ckpt, ctx->L.f_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+            rs = record_steps(ctx, len, uhist);
+        } else if (s > 0) {
+            rs = record_march(ctx, ckpt, len, uhist);
+        } else {
+            LBRS_CUDA(ctx, launch_pull_into(ctx, ckpt, uhist));
+            rs = record_march(ctx, uhist, len - 1, uhist + ustride);
+        }
         if (rs != LBRS_OK) return rs;
         if (fused2_f32(ctx)) {
             // sweep on k = fbar: k^{end} from g^{end}, two steps per launch while U_{s-1} and
@@ -1623,8 +1810,11 @@ lbrs_status lbrs_backward_checkpointed(lbrs_ctx* ctx, void* d_adj_ws, const void
     LBRS_CUDA(ctx, launch_vjp_eq_raw(ctx, uhist, g[gc], d_gradU0));
     ctx->launches += 2;
     // restore the final forward state
-    LBRS_CUDA(ctx, cudaMemcpyAsync(ctx->f[ctx->cur], ws + A.ckpt0 + A.nseg * A.ckpt_stride, ctx->L.f_bytes,
-                                   cudaMemcpyDeviceToDevice, ctx->stream));
+    const char* final_state = ws + A.ckpt0 + A.nseg * A.ckpt_stride;
+    if (ctx->adj_moments)
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, final_state));
+    else
+        LBRS_CUDA(ctx, cudaMemcpyAsync(ctx->f[ctx->cur], final_state, ctx->L.f_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
     ctx->step = ctx->adj_step0 + ctx->adj_n;
     return LBRS_OK;
 }

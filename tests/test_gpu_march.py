@@ -1,0 +1,62 @@
+"""The marching kernel (FP32 D2Q4 at omega = 1 on the moments, two steps a launch) against one storing
+step a launch: bit-identical distributions, moments and recorded moments.
+
+Grids sit at the edges of the kernel's 60-column strips and 64-column windows, of its rows per warp and
+of the rows beside a y side; sides of every kind it takes.  The two paths run in processes of their own
+(the switches are read once per process)."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+_SCRIPT = r"""
+import sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np
+import torch
+from paper_1504_07034_gb300.solver import Solver
+
+D0, D1 = (0.9, 0.6, -0.2, 0.8), (1.1, -0.3, 0.4, 1.2)
+T, P, WL = ("transmissive", None), ("periodic", None), ("wall", None)
+SETS = [[P, P, P, P], [T, T, T, T], [("dirichlet", D0), T, WL, ("dirichlet", D1)], [P, P, WL, WL],
+        [T, ("dirichlet", D1), ("dirichlet", D0), WL], [("dirichlet", D1), ("dirichlet", D0), P, P],
+        [("dirichlet", D0), ("dirichlet", D1), T, ("dirichlet", D0)]]
+SHAPES = [(1, 1), (2, 3), (59, 2), (60, 5), (61, 4), (62, 7), (63, 9), (64, 33), (65, 40), (119, 6), (120, 64),
+          (121, 17), (257, 70), (1021, 13), (1200, 131)]
+rng = np.random.default_rng(7)
+out = []
+for bc in SETS:
+    for nx, ny in SHAPES:
+        if "wall" in (bc[2][0], bc[3][0]) and ny < 2:
+            continue
+        W = np.stack([rng.uniform(0.3, 1.5, (ny, nx)), rng.uniform(-0.8, 0.8, (ny, nx)),
+                      rng.uniform(-0.8, 0.8, (ny, nx)), rng.uniform(0.2, 1.5, (ny, nx))])
+        for precision in ("f32", "f32u"):
+            s = Solver("d2q4", nx, ny, lam=7.0, dx=0.01, bc=bc, omega=1.0, precision=precision)
+            s.set_state(torch.from_numpy(W).cuda())
+            for n in (1, 2, 6, 7, 70):           # single launches, and a captured graph with a remainder
+                s.step(n)
+                out.append(s.raw_state().cpu().numpy().view(np.float32).ravel())
+            if precision == "f32":
+                out.append(s.step_record(5).cpu().numpy().ravel())
+                out.append(s.raw_state().cpu().numpy().view(np.float32).ravel())
+            s.close()
+np.save(sys.argv[2], np.concatenate(out))
+"""
+
+
+def test_march_equals_single_steps(tmp_path):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    script = tmp_path / "march.py"
+    script.write_text(_SCRIPT)
+    res = {}
+    for name, env in (("march", {}), ("single", {"LBRS_F32_MARCH": "0", "LBRS_F32_FUSE": "0", "LBRS_F32U_FUSE": "0"})):
+        out = tmp_path / f"{name}.npy"
+        subprocess.run([sys.executable, str(script), root, str(out)], check=True, env=dict(os.environ, **env), timeout=600)
+        res[name] = np.load(out)
+    assert np.all(np.isfinite(res["single"]))
+    assert np.array_equal(res["march"], res["single"]), np.max(np.abs(res["march"] - res["single"]))
