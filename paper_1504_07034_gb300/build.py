@@ -1,12 +1,13 @@
 """Build the LBRS CUDA library (liblbrs.so) in-tree for sm_103a.
 
-Seven translation units compiled in parallel with nvcc, then linked into one
+Eight translation units compiled in parallel with nvcc, then linked into one
 shared library with the CUDA runtime linked statically:
 
   csrc/lbrs_kernels_f64.cu  FP64 kernels, -fmad=false (rounding as written)
   csrc/lbrs_kernels_f32.cu  FP32 step kernels
   csrc/lbrs_kernels_f16.cu  D2Q4 step with FP16 non-equilibrium storage
   csrc/lbrs_kernels_march.cu FP32 D2Q4 steps at omega = 1 on the moments
+  csrc/lbrs_kernels_tube.cu FP32 1-D tubes in registers
   csrc/lbrs_runtime.cu      host C ABI (include/lbrs.h)
   csrc/lbrs_noalloc.cu      diagnostics variant with static scratch, -fmad=false
   csrc/lbrs_batch_runtime.cu host runtime of the batched tubes
@@ -43,11 +44,12 @@ UNITS = {
     "lbrs_kernels_f32.cu": [],
     "lbrs_kernels_f16.cu": [],
     "lbrs_kernels_march.cu": [],
+    "lbrs_kernels_tube.cu": [],
     "lbrs_runtime.cu": [],
     "lbrs_noalloc.cu": ["-fmad=false"],
     "lbrs_batch_runtime.cu": [],
 }
-HEADERS = [CSRC / "lbrs_kernels.cuh", CSRC / "lbrs_batch.cuh", CSRC / "lbrs_march.cuh", CSRC / "lbrs_launch.h", INCLUDE / "lbrs.h"]
+HEADERS = [CSRC / "lbrs_kernels.cuh", CSRC / "lbrs_batch.cuh", CSRC / "lbrs_march.cuh", CSRC / "lbrs_tube.cuh", CSRC / "lbrs_launch.h", INCLUDE / "lbrs.h"]
 
 
 def nvcc() -> str:

@@ -445,6 +445,79 @@ __global__ void adapt_prep_kernel(AdaptState* st, Ts* ghost, GhostSpec g, double
     st->last = next_last;
 }
 
+// FP64 D1Q2 / D1Q3 tube, several steps per launch with the populations in registers: one block per
+// tile steps a window of 32 kTubeWarps64 cells, one a thread, `halo` of them beyond the tile each
+// side; neighbours by shuffles, across warps through shared memory with one barrier a step.  Bound by
+// the chain of dependent FP64 operations of a step (about 60 of them), hence one cell a thread and as
+// many steps a launch as the window allows.  Per cell the operations are step1d_kernel's, in its order;
+// U/3 (D1Q3) by the reciprocal's product and one correction of the remainder (Markstein), which rounds
+// as the division does.
+constexpr int kTubeWarps64 = 4, kTubeWin64 = 32 * kTubeWarps64;
+
+template <int Q, bool OM1>
+__global__ void __launch_bounds__(kTubeWin64) tube1d_f64_kernel(const StepArgs<double> a, int steps, int halo, int ntiles)
+{
+    __shared__ double s_l[2][kTubeWarps64][3], s_r[2][kTubeWarps64][3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nx = a.nx, tile = blockIdx.x;
+    const int t0 = (int)((int64_t)tile * nx / ntiles), t1 = (int)((int64_t)(tile + 1) * nx / ntiles);
+    const int x = t0 - halo + (int)threadIdx.x;
+    const bool per = a.bc[0] == BC_PERIODIC;
+    const bool first = !per && x == 0, last = !per && x == nx - 1;
+    int xm = min(max(x, 0), nx - 1);
+    if (per) {
+        xm = x % nx;
+        if (xm < 0) xm += nx;
+    }
+    double f[Q][3];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f[q][k] = a.src[LBRS_IX((q * 3 + k) * a.N + xm, 3 * Q * a.N, 55)];
+    // what the tube's ends pull: a Dirichlet side's ghost, else their own population
+    const bool gfirst = first && a.bc[0] == BC_DIRICHLET, glast = last && a.bc[1] == BC_DIRICHLET;
+    double gl[3] = {0.0, 0.0, 0.0}, gr[3] = {0.0, 0.0, 0.0};
+    if (gfirst)
+        for (int k = 0; k < 3; ++k) gr[k] = a.ghost[3 * (Q - 1) + k];
+    if (glast)
+        for (int k = 0; k < 3; ++k) gl[k] = a.ghost[GHOST_STRIDE + k];
+    for (int s = 0; s < steps; ++s) {
+        const int b = s & 1;
+        if (lane == 0)
+            for (int k = 0; k < 3; ++k) s_l[b][warp][k] = f[0][k];
+        if (lane == 31)
+            for (int k = 0; k < 3; ++k) s_r[b][warp][k] = f[Q - 1][k];
+        __syncthreads();
+        double in[Q][3], U[3], e[Q][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            double r = __shfl_up_sync(0xffffffffu, f[Q - 1][k], 1);
+            double l = __shfl_down_sync(0xffffffffu, f[0][k], 1);
+            if (lane == 0 && warp > 0) r = s_r[b][warp - 1][k];
+            if (lane == 31 && warp < kTubeWarps64 - 1) l = s_l[b][warp + 1][k];
+            if (first) r = gfirst ? gr[k] : f[Q - 1][k];
+            if (last) l = glast ? gl[k] : f[0][k];
+            in[0][k] = l;
+            if constexpr (Q == 3) in[1][k] = f[1][k];
+            in[Q - 1][k] = r;
+            U[k] = Q == 3 ? (in[0][k] + in[1][k]) + in[Q - 1][k] : in[0][k] + in[Q - 1][k];
+        }
+        if constexpr (Q == 3) {
+            equilibria1d3<double>(U, a.gm1, a.c, e);
+        } else {
+            equilibria1d<double>(U, a.gm1, a.c, e);
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) f[q][k] = OM1 ? e[q][k] : a.om1 * in[q][k] + a.om * e[q][k];
+    }
+    if (x < t0 || x >= t1) return;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) a.dst[LBRS_IX((q * 3 + k) * a.N + x, 3 * Q * a.N, 55)] = f[q][k];
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
@@ -811,6 +884,28 @@ cudaError_t launch_adapt_step_f64(const StepArgs<double>& a, void* st, double ga
 cudaError_t launch_adapt_init_bound_f64(const void* fs, int64_t N, double gamma, void* st, cudaStream_t s)
 {
     adapt_init_bound_kernel<double><<<grid_for(N), 256, 0, s>>>((const double*)fs, N, gamma, (AdaptState*)st);
+    return cudaGetLastError();
+}
+
+// Steps per launch (the window's halo): more of them leave less of the 128-cell window to the tile;
+// as many as keep one block per SM, within which a block takes as long as a lone one (480 D1Q2 steps:
+// 1000 cells 611 us at 48 steps a launch, 631 at 32, 693 at 16; 8000 cells 1041, 632, 693; 20000 cells
+// 2515, 1546, 1123 and at 24 steps 1082; one step a launch 2600 to 2720).
+int tube_f64_steps(int64_t nx)
+{
+    for (int h : {48, 32, 24})
+        if (nx <= 152 * (kTubeWin64 - 2 * h)) return h;
+    return 16;
+}
+
+cudaError_t launch_tube_f64(int q, const StepArgs<double>& a, int steps, cudaStream_t s)
+{
+    const int halo = tube_f64_steps(a.nx), tile = kTubeWin64 - 2 * halo, n = (a.nx + tile - 1) / tile;
+    const bool om1 = a.om1 == 0.0;
+    if (q == 3 && om1) tube1d_f64_kernel<3, true><<<n, kTubeWin64, 0, s>>>(a, steps, halo, n);
+    else if (q == 3) tube1d_f64_kernel<3, false><<<n, kTubeWin64, 0, s>>>(a, steps, halo, n);
+    else if (om1) tube1d_f64_kernel<2, true><<<n, kTubeWin64, 0, s>>>(a, steps, halo, n);
+    else tube1d_f64_kernel<2, false><<<n, kTubeWin64, 0, s>>>(a, steps, halo, n);
     return cudaGetLastError();
 }
 

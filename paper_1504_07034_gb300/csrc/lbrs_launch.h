@@ -37,6 +37,7 @@ unsigned long long debug_word_f32(int clear);
 unsigned long long debug_word_f64(int clear);
 unsigned long long debug_word_f16(int clear);
 unsigned long long debug_word_march(int clear);
+unsigned long long debug_word_tube(int clear);
 
 // Failure-detection self-test: a bounded wait on an mbarrier that nothing completes
 // gives up and raises *wait_flag (one block, 4096 polls).
@@ -166,6 +167,19 @@ cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaSt
 // From stored distributions (a.src) the moments U of the next step, and f* = f^eq(U) back.
 cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s);
 cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s);
+
+// FP32 1-D tubes in registers (lbrs_tube.cuh, lbrs_kernels_tube.cu), up to kTubeMaxHalo steps a
+// launch: batched ones in tiles of at most tube_tile_cells cells (0: not for this halo), of which
+// every tile of a tube with more than one holds at least half as many; and a tube by itself.
+constexpr int kTubeMaxHalo = 64;
+int tube_tile_cells(int halo, bool omega1);
+cudaError_t launch_tubes_f32(const BatchArgs<float>& a, int ntiles, cudaStream_t s);
+cudaError_t launch_one_tube_f32(const BatchArgs<float>& a, cudaStream_t s);
+
+// FP64 D1Q2 (q = 2) / D1Q3 tube, any end conditions: `steps` <= tube_f64_steps(nx) steps in one launch,
+// bit-identical to single ones.
+int tube_f64_steps(int64_t nx);
+cudaError_t launch_tube_f64(int q, const StepArgs<double>& a, int steps, cudaStream_t s);
 
 // Batched D1Q2 / D1Q3 tubes with temporal blocking (lbrs_batch.cuh): one CTA of
 // `block` threads per active tile; dynamic shared memory 2*3Q*(TILE+2H) elements.

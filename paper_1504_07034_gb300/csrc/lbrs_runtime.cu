@@ -294,25 +294,26 @@ cudaError_t launch_one_step(lbrs_ctx* ctx, int from, cudaStream_t s)
     return launch_step_f32(lat, step_args<float>(ctx, from), s);
 }
 
-// FP32 1-D (D1Q2, D1Q3) with both ends transmissive or both periodic: steps taken by the batched
-// tubes' temporal-blocking kernel as a tube of one, up to kOneHalo steps per launch in shared memory
-// (tiles of 4 kOneBlock - 2 kOneHalo cells; the single-tube arithmetic, bit-identical to one step a
-// launch).  LBRS_1D_BLOCKED=0 keeps one step a launch.
-constexpr int kOneBlock = 256, kOneCellsPerThread = 4, kOneHalo = 32;
-constexpr int kOneTile = kOneBlock * kOneCellsPerThread - 2 * kOneHalo;
+// FP32 1-D (D1Q2, D1Q3) with both ends transmissive or both periodic: up to kOneHalo steps per launch
+// by the tubes' register kernel (lbrs_tube.cuh; the single-tube arithmetic, bit-identical to one step
+// a launch).  LBRS_1D_BLOCKED=0 keeps one step a launch.
+constexpr int kOneHalo = 32;
 
-bool blocked_1d(const lbrs_ctx* ctx)
+bool blocked_1d_enabled()
 {
     static const int enabled = [] {
         const char* e = getenv("LBRS_1D_BLOCKED");
         return (e && !strcmp(e, "0")) ? 0 : 1;
     }();
-    if (!enabled || ctx->f64 || (ctx->lattice != LBRS_D1Q2 && ctx->lattice != LBRS_D1Q3)) return false;
+    return enabled != 0;
+}
+
+bool blocked_1d(const lbrs_ctx* ctx)
+{
+    if (!blocked_1d_enabled() || ctx->f64 || (ctx->lattice != LBRS_D1Q2 && ctx->lattice != LBRS_D1Q3)) return false;
     const int k0 = ctx->cfg.bc[0].kind, k1 = ctx->cfg.bc[1].kind;
     return k0 == k1 && (k0 == LBRS_BC_TRANSMISSIVE || k0 == LBRS_BC_PERIODIC);
 }
-
-size_t blocked_1d_smem(const lbrs_ctx* ctx) { return 2 * 3 * (size_t)ctx->Q * (kOneTile + 2 * kOneHalo) * sizeof(float); }
 
 // m <= kOneHalo steps of a blocked 1-D context from buffer `from` in one launch.
 cudaError_t launch_blocked_1d(const lbrs_ctx* ctx, int from, int m, cudaStream_t s)
@@ -322,7 +323,6 @@ cudaError_t launch_blocked_1d(const lbrs_ctx* ctx, int from, int m, cudaStream_t
     a.dst = (float*)ctx->f[from ^ 1];
     a.N = ctx->N;
     a.tiles = nullptr;
-    a.tile_cells = kOneTile;
     a.halo = kOneHalo;
     a.periodic = ctx->cfg.bc[0].kind == LBRS_BC_PERIODIC;
     a.launch = 0;
@@ -333,11 +333,7 @@ cudaError_t launch_blocked_1d(const lbrs_ctx* ctx, int from, int m, cudaStream_t
     a.one_len = (int)ctx->cfg.nx;
     a.one_steps = m;
     a.one_c = (float)ctx->c;
-    const int ntiles = (int)((ctx->cfg.nx + kOneTile - 1) / kOneTile);
-    // the kernel's shared-memory limit is shared with the batched tubes, which set it per tuning
-    const cudaError_t e = prepare_batch_f32(kOneBlock, blocked_1d_smem(ctx), ctx->Q);
-    if (e != cudaSuccess) return e;
-    return launch_batch_f32(a, ntiles, kOneBlock, s);
+    return launch_one_tube_f32(a, s);
 }
 
 // The FP32 distribution form's two-steps-per-launch kernel available for this context?
@@ -825,7 +821,8 @@ lbrs_status lbrs_debug_check(uint64_t* first)
 {
     if (!first) return fail(nullptr, LBRS_EINVAL, "first is NULL");
     unsigned long long w = 0ull;
-    for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1), debug_word_march(1)})
+    for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1), debug_word_march(1),
+                                 debug_word_tube(1)})
         if (!w) w = v;
     *first = (uint64_t)w;
     if (w)
@@ -901,7 +898,9 @@ lbrs_status lbrs_create(const lbrs_config* cfg, void* d_workspace, size_t bytes,
         for (int k = 0; k < 4; ++k) g.prim[s][k] = cfg->bc[s].prim[k];
     }
     ctx->gspec = g;
-    if (cfg->lattice == LBRS_D2Q4) march_ghosts(g, cfg->gamma, ctx->c, ctx->mghost);
+    if (cfg->lattice == LBRS_D2Q4) {
+        march_ghosts(g, cfg->gamma, ctx->c, ctx->mghost);
+    }
     const int lat = lat_code(cfg->lattice);
     cudaError_t e = launch_ghost(lat, ctx->f64, g, cfg->gamma, ctx->c, ctx->ws + L.ghost, ctx->stream);
     if (e != cudaSuccess) {
@@ -1003,6 +1002,12 @@ lbrs_status lbrs_step(lbrs_ctx* ctx, int64_t n)
     return LBRS_OK;
 }
 
+// FP64 1-D: several steps per launch in registers; LBRS_1D_BLOCKED=0 keeps one.
+static bool tube_f64(const lbrs_ctx* ctx)
+{
+    return blocked_1d_enabled() && ctx->f64 && (ctx->lattice == LBRS_D1Q2 || ctx->lattice == LBRS_D1Q3);
+}
+
 // n steps at omega = 1 on the moments.  Distribution storage enters through the pull of the first
 // step and leaves through the equilibria of the last, back into the buffer it came from.
 static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
@@ -1049,6 +1054,17 @@ static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
         for (int64_t left = n; left > 0;) {
             const int m = (int)(left < kOneHalo ? left : kOneHalo);
             LBRS_CUDA(ctx, launch_blocked_1d(ctx, ctx->cur, m, ctx->stream));
+            ctx->cur ^= 1;
+            ctx->step += m;
+            ctx->launches += 1;
+            left -= m;
+        }
+        return LBRS_OK;
+    }
+    if (tube_f64(ctx)) {
+        for (int64_t left = n; left > 0;) {
+            const int most = tube_f64_steps(ctx->cfg.nx), m = (int)(left < most ? left : most);
+            LBRS_CUDA(ctx, launch_tube_f64(ctx->Q, step_args<double>(ctx, ctx->cur), m, ctx->stream));
             ctx->cur ^= 1;
             ctx->step += m;
             ctx->launches += 1;
