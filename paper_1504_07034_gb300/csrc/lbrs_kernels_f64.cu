@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "lbrs_kernels.cuh"
+#include "lbrs_fp64.cuh"
 #include "lbrs_batch.cuh"
 #include "lbrs_launch.h"
 
