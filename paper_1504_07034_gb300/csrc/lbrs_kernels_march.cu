@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
 // takes the minimum over the rows (1024^2: 16 rows 10.1 us, 8 rows 11.0, 30 rows 15.3; 4096 x 1024:
 // 30 rows 29.3, 12 rows 31.8).  The warps beside y sides that are not periodic take longer per row
 // (0.40 us by themselves, 0.60 beside a wall) and get as many rows as keep them from ending last.
-void march_rows_for(MarchArgs& a, int own, int steps)
+// Returns that time.
+double march_rows_for(MarchArgs& a, int own, int steps)
 {
     a.strips = (a.nx + own - 1) / own;
     const bool per = a.bc[2] == BC_PERIODIC;
@@ -118,6 +119,7 @@ void march_rows_for(MarchArgs& a, int own, int steps)
             a.chunks = (int)chunks;
         }
     }
+    return best;
 }
 
 template <int K, bool RECORD>
@@ -132,13 +134,33 @@ cudaError_t launch_k(MarchArgs a, cudaStream_t s)
 
 }  // namespace
 
-bool march_enabled()
+static int march_mode()
 {
     static const int v = [] {
         const char* e = getenv("LBRS_F32_MARCH");
-        return (e && !strcmp(e, "0")) ? 0 : 1;
+        return e ? atoi(e) : 1;
     }();
-    return v != 0;
+    return v;
+}
+
+bool march_enabled() { return march_mode() != 0; }
+
+// The tile kernel's two-step launch (step2d_u2_kernel, 32 x 16 tiles, four blocks per SM) starts
+// faster than a march and wins on small grids: about 2.7 us and 1.05 us per tile of an SM against the
+// march's 3 us and its own time, a quarter more of it beside sides that are not periodic (per launch,
+// in a graph: 128^2 3.7 against 4.4 us periodic and 5.4 with clamped sides, 384^2 4.5 against 5.6 and
+// 6.5, 512^2 6.7 against 5.6 and 6.6, 1531 x 200 6.9 against 6.4 and 10.0, 768^2 10.7 against 7.9 and
+// 8.8).
+bool march_prefers_tiles(int nx, int ny, const int bc[4])
+{
+    if (march_mode() >= 2) return false;
+    MarchArgs a;
+    a.nx = nx;
+    a.ny = ny;
+    for (int s = 0; s < 4; ++s) a.bc[s] = bc[s];
+    const double march = 3.0 + march_rows_for(a, MarchShape<2>::own, 2) * (bc[2] == BC_PERIODIC ? 1.0 : 1.25);
+    const double tiles = (double)((nx + 31) / 32) * (double)((ny + 15) / 16);
+    return 2.7 + 1.05 * tiles / kSMs < march;
 }
 
 // f^eq of the Dirichlet sides' states in FP64, rounded: the values of the device's ghost table

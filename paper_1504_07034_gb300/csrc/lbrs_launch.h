@@ -161,6 +161,9 @@ struct MarchStep {
     float c, gm1;
 };
 bool march_enabled();
+// The moments-only form's tile kernels (launch_step2_f32u) are faster on this grid; never with
+// LBRS_F32_MARCH=2.
+bool march_prefers_tiles(int nx, int ny, const int bc[4]);
 
 void march_ghosts(const GhostSpec& g, double gamma, double c, float out[4][16]);
 cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaStream_t s);

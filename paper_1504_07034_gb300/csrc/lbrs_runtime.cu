@@ -130,6 +130,7 @@ struct lbrs_ctx {
     const uint8_t* solid;    // caller-owned obstacle mask [ny][nx] (lbrs_set_obstacles), or NULL
     cudaGraphExec_t mgraph[2];   // kGraphSteps steps on the moments held in buffer b
     float mghost[4][16];     // the march's copy of the ghost table
+    bool mtiles;             // steps on the moments run on tiles (small grids), not by the march
     GhostSpec gspec;         // the sides' kinds and states (the adaptive run rebuilds the ghosts)
     bool adapt_ready;        // the adaptive record holds the current state's run
     bool adapt_used;         // the distributions carry an adaptive lambda
@@ -398,9 +399,20 @@ MarchStep march_step(const lbrs_ctx* ctx, const char* src, char* dst)
     return m;
 }
 
+// m = 1 or 2 steps on the moments from src into dst.
+cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int m, cudaStream_t s)
+{
+    if (!ctx->mtiles) return launch_march_f32(march_step(ctx, src, dst), m, false, s);
+    F16StepArgs a = f16_args(ctx, 0);
+    a.src = src;
+    a.dst = dst;
+    return m == 2 ? launch_step2_f32u(a, s) : launch_step_f32u(a, s);
+}
+
 // Distribution storage enters and leaves the moments once per call (80 + 80 B per cell, two
-// launches): worth it from this many steps on (1024^2: 6 steps in 52 us instead of 80 us).
-constexpr int64_t kMarchMin = 6;
+// launches): worth it from this many steps on (1024^2: 6 steps in 45 us instead of 80 us; 128^2:
+// 8 steps in 37 us instead of 41, 6 in 33 instead of 30).
+int64_t march_min(const lbrs_ctx* ctx) { return ctx->N < 400000 ? 8 : 6; }
 
 // Steps the next launch takes out of `left`: three where the three-step kernel applies (but
 // 2 + 2 rather than 3 + 1), else two where the two-step kernel does, else one.
@@ -455,7 +467,7 @@ cudaError_t launch_march_run(const lbrs_ctx* ctx, char* const v[2], int64_t n, c
     int b = 0;
     for (; n > 0; b ^= 1, ++*launches) {
         const int m = n >= 2 ? 2 : 1;
-        const cudaError_t e = launch_march_f32(march_step(ctx, v[b], v[b ^ 1]), m, false, s);
+        const cudaError_t e = launch_u_steps(ctx, v[b], v[b ^ 1], m, s);
         if (e != cudaSuccess) return e;
         n -= m;
     }
@@ -716,7 +728,7 @@ cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U)
 lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
 {
     const size_t stride = (size_t)ctx->K * ctx->N * elem_bytes(ctx);
-    if (march(ctx) && n >= kMarchMin) {
+    if (march(ctx) && n >= march_min(ctx)) {
         LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], U_hist));
         lbrs_status st = record_march(ctx, U_hist, n - 1, U_hist + stride);
         if (st != LBRS_OK) return st;
@@ -900,6 +912,9 @@ lbrs_status lbrs_create(const lbrs_config* cfg, void* d_workspace, size_t bytes,
     ctx->gspec = g;
     if (cfg->lattice == LBRS_D2Q4) {
         march_ghosts(g, cfg->gamma, ctx->c, ctx->mghost);
+        int kinds[4];
+        for (int s = 0; s < 4; ++s) kinds[s] = kernel_bc(ctx, s);
+        ctx->mtiles = march_prefers_tiles((int)cfg->nx, (int)ctx->ny_store, kinds);
     }
     const int lat = lat_code(cfg->lattice);
     cudaError_t e = launch_ghost(lat, ctx->f64, g, cfg->gamma, ctx->c, ctx->ws + L.ghost, ctx->stream);
@@ -1074,7 +1089,7 @@ static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
     }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBRS_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
-    if (march(ctx) && (ctx->f32u || n >= kMarchMin)) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
+    if (march(ctx) && (ctx->f32u || n >= march_min(ctx))) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
     int64_t left = n;
     const int G = graph_steps(ctx);
     if (cap == cudaStreamCaptureStatusNone && n >= 2 * G) {
@@ -1724,7 +1739,7 @@ lbrs_status lbrs_forward_checkpointed(lbrs_ctx* ctx, int64_t n_steps, int64_t se
                 if (done == 0) {
                     LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], to));
                 } else {
-                    LBRS_CUDA(ctx, launch_march_f32(march_step(ctx, at, to), m, false, ctx->stream));
+                    LBRS_CUDA(ctx, launch_u_steps(ctx, at, to, m, ctx->stream));
                     ctx->launches += 1;
                 }
                 at = to;

@@ -2,8 +2,9 @@
 step a launch: bit-identical distributions, moments and recorded moments.
 
 Grids sit at the edges of the kernel's 60-column strips and 64-column windows, of its rows per warp and
-of the rows beside a y side; sides of every kind it takes.  The two paths run in processes of their own
-(the switches are read once per process)."""
+of the rows beside a y side; sides of every kind it takes.  Small grids step
+on the moments-only form's tiles by default, so the march is also run on all of them
+(LBRS_F32_MARCH=2).  The paths run in processes of their own (the switches are read once per process)."""
 import os
 import subprocess
 import sys
@@ -38,11 +39,11 @@ for bc in SETS:
         for precision in ("f32", "f32u"):
             s = Solver("d2q4", nx, ny, lam=7.0, dx=0.01, bc=bc, omega=1.0, precision=precision)
             s.set_state(torch.from_numpy(W).cuda())
-            for n in (1, 2, 6, 7, 70):           # single launches, and a captured graph with a remainder
+            for n in (1, 2, 8, 9, 70):           # single launches, and a captured graph with a remainder
                 s.step(n)
                 out.append(s.raw_state().cpu().numpy().view(np.float32).ravel())
             if precision == "f32":
-                out.append(s.step_record(5).cpu().numpy().ravel())
+                out.append(s.step_record(9).cpu().numpy().ravel())
                 out.append(s.raw_state().cpu().numpy().view(np.float32).ravel())
             s.close()
 np.save(sys.argv[2], np.concatenate(out))
@@ -54,9 +55,10 @@ def test_march_equals_single_steps(tmp_path):
     script = tmp_path / "march.py"
     script.write_text(_SCRIPT)
     res = {}
-    for name, env in (("march", {}), ("single", {"LBRS_F32_MARCH": "0", "LBRS_F32_FUSE": "0", "LBRS_F32U_FUSE": "0"})):
+    for name, env in (("march", {"LBRS_F32_MARCH": "2"}), ("default", {}), ("single", {"LBRS_F32_MARCH": "0", "LBRS_F32_FUSE": "0", "LBRS_F32U_FUSE": "0"})):
         out = tmp_path / f"{name}.npy"
         subprocess.run([sys.executable, str(script), root, str(out)], check=True, env=dict(os.environ, **env), timeout=600)
         res[name] = np.load(out)
     assert np.all(np.isfinite(res["single"]))
-    assert np.array_equal(res["march"], res["single"]), np.max(np.abs(res["march"] - res["single"]))
+    for name in ("march", "default"):
+        assert np.array_equal(res[name], res["single"]), (name, np.max(np.abs(res[name] - res["single"])))
