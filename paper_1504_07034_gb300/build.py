@@ -1,6 +1,6 @@
 """Build the LBRS CUDA library (liblbrs.so) in-tree for sm_103a.
 
-Eight translation units compiled in parallel with nvcc, then linked into one
+Nine translation units compiled in parallel with nvcc, then linked into one
 shared library with the CUDA runtime linked statically:
 
   csrc/lbrs_kernels_f64.cu  FP64 kernels, -fmad=false (rounding as written)
@@ -8,6 +8,7 @@ shared library with the CUDA runtime linked statically:
   csrc/lbrs_kernels_f16.cu  D2Q4 step with FP16 non-equilibrium storage
   csrc/lbrs_kernels_march.cu FP32 D2Q4 steps at omega = 1 on the moments
   csrc/lbrs_kernels_tube.cu FP32 1-D tubes in registers
+  csrc/lbrs_kernels_scalar.cu FP32 scalar D2Q4 steps in shared-memory windows
   csrc/lbrs_runtime.cu      host C ABI (include/lbrs.h)
   csrc/lbrs_noalloc.cu      diagnostics variant with static scratch, -fmad=false
   csrc/lbrs_batch_runtime.cu host runtime of the batched tubes
@@ -45,12 +46,13 @@ UNITS = {
     "lbrs_kernels_f16.cu": [],
     "lbrs_kernels_march.cu": [],
     "lbrs_kernels_tube.cu": [],
+    "lbrs_kernels_scalar.cu": [],
     "lbrs_runtime.cu": [],
     "lbrs_noalloc.cu": ["-fmad=false"],
     "lbrs_batch_runtime.cu": [],
 }
 HEADERS = [CSRC / "lbrs_kernels.cuh", CSRC / "lbrs_batch.cuh", CSRC / "lbrs_march.cuh", CSRC / "lbrs_tube.cuh",
-           CSRC / "lbrs_fp64.cuh", CSRC / "lbrs_launch.h", INCLUDE / "lbrs.h"]
+           CSRC / "lbrs_scalar.cuh",            CSRC / "lbrs_fp64.cuh", CSRC / "lbrs_launch.h", INCLUDE / "lbrs.h"]
 
 
 def nvcc() -> str:

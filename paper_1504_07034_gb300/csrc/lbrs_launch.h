@@ -38,6 +38,7 @@ unsigned long long debug_word_f64(int clear);
 unsigned long long debug_word_f16(int clear);
 unsigned long long debug_word_march(int clear);
 unsigned long long debug_word_tube(int clear);
+unsigned long long debug_word_scalar(int clear);
 
 // Failure-detection self-test: a bounded wait on an mbarrier that nothing completes
 // gives up and raises *wait_flag (one block, 4096 polls).
@@ -170,6 +171,21 @@ cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaSt
 // From stored distributions (a.src) the moments U of the next step, and f* = f^eq(U) back.
 cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s);
 cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s);
+
+// Scalar D2Q4 in FP32 at omega = 1 on the field u in shared-memory windows (lbrs_scalar.cuh,
+// lbrs_kernels_scalar.cu), bit-identical to single steps; off when LBRS_F32S_WINDOW=0.  Not for
+// Dirichlet x sides beside periodic y sides (whose corner profile depends on the unwrapped row).
+struct ScalarPlan {
+    int wx, wy, hx, hy, tx, ty;   // window, cells beyond the tile, tile
+    int rows;                     // rows a thread owns
+    int steps;                    // steps per launch at most
+};
+bool scalar_windows_enabled();
+ScalarPlan scalar_plan(int nx, int ny, const int bc[4]);
+// steps <= plan.steps; loadf: from the distributions f.src, whose pull comes on top (one step more);
+// else from u.  storef: f* to dst, else u.
+cudaError_t launch_scalar_window(const StepArgs<float>& f, const ScalarPlan& p, const float* u, float* dst, int steps,
+                                 bool loadf, bool storef, cudaStream_t s);
 
 // FP32 1-D tubes in registers (lbrs_tube.cuh, lbrs_kernels_tube.cu), up to kTubeMaxHalo steps a
 // launch: batched ones in tiles of at most tube_tile_cells cells (0: not for this halo), of which

@@ -130,6 +130,7 @@ struct lbrs_ctx {
     const uint8_t* solid;    // caller-owned obstacle mask [ny][nx] (lbrs_set_obstacles), or NULL
     cudaGraphExec_t mgraph[2];   // kGraphSteps steps on the moments held in buffer b
     float mghost[4][16];     // the march's copy of the ghost table
+    ScalarPlan splan;        // scalar lattice: windows of the steps on u (steps = 0: not used)
     bool mtiles;             // steps on the moments run on tiles (small grids), not by the march
     GhostSpec gspec;         // the sides' kinds and states (the adaptive run rebuilds the ghosts)
     bool adapt_ready;        // the adaptive record holds the current state's run
@@ -834,7 +835,7 @@ lbrs_status lbrs_debug_check(uint64_t* first)
     if (!first) return fail(nullptr, LBRS_EINVAL, "first is NULL");
     unsigned long long w = 0ull;
     for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1), debug_word_march(1),
-                                 debug_word_tube(1)})
+                                 debug_word_tube(1), debug_word_scalar(1)})
         if (!w) w = v;
     *first = (uint64_t)w;
     if (w)
@@ -910,6 +911,13 @@ lbrs_status lbrs_create(const lbrs_config* cfg, void* d_workspace, size_t bytes,
         for (int k = 0; k < 4; ++k) g.prim[s][k] = cfg->bc[s].prim[k];
     }
     ctx->gspec = g;
+    if (cfg->lattice == LBRS_D2Q4S && !ctx->f64 && cfg->omega == 1.0 && scalar_windows_enabled() && fused2_scalar(ctx) &&
+        !(cfg->bc[2].kind == LBRS_BC_PERIODIC &&
+          (cfg->bc[0].kind == LBRS_BC_DIRICHLET || cfg->bc[1].kind == LBRS_BC_DIRICHLET))) {
+        int kinds[4];
+        for (int s = 0; s < 4; ++s) kinds[s] = kernel_bc(ctx, s);
+        ctx->splan = scalar_plan((int)cfg->nx, (int)cfg->ny, kinds);
+    }
     if (cfg->lattice == LBRS_D2Q4) {
         march_ghosts(g, cfg->gamma, ctx->c, ctx->mghost);
         int kinds[4];
@@ -1063,8 +1071,34 @@ static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
     return LBRS_OK;
 }
 
+// n >= 2 scalar steps at omega = 1 on u: the first launch pulls from the distributions, the last
+// leaves them; u stays in the idle buffer between (where one launch does, it writes there and the
+// buffers change places).
+static lbrs_status step_scalar(lbrs_ctx* ctx, int64_t n)
+{
+    const StepArgs<float> f = step_args<float>(ctx, ctx->cur);
+    float* const v[2] = {(float*)ctx->f[ctx->cur ^ 1], (float*)ctx->f[ctx->cur ^ 1] + ctx->N};
+    const float* u = nullptr;
+    int b = 0;
+    for (int64_t left = n; left > 0;) {
+        const bool first = left == n;
+        const int64_t most = ctx->splan.steps + (first ? 1 : 0), m = left < most ? left : most;
+        const bool last = m == left;
+        float* dst = !last ? v[b] : (first ? v[0] : (float*)ctx->f[ctx->cur]);
+        LBRS_CUDA(ctx, launch_scalar_window(f, ctx->splan, u, dst, (int)(first ? m - 1 : m), first, last, ctx->stream));
+        ctx->launches += 1;
+        if (first && last) ctx->cur ^= 1;
+        u = dst;
+        b ^= 1;
+        left -= m;
+    }
+    ctx->step += n;
+    return LBRS_OK;
+}
+
 static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
 {
+    if (ctx->splan.steps && n >= 2) return step_scalar(ctx, n);
     if (blocked_1d(ctx)) {
         for (int64_t left = n; left > 0;) {
             const int m = (int)(left < kOneHalo ? left : kOneHalo);
