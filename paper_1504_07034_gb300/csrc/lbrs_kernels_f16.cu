@@ -48,6 +48,7 @@ struct F16Args {
     int nx, ny;
     int bc[4];
     float om, om1, c, gm1;
+    const uint8_t* __restrict__ walls; // two-step kernel with internal walls: [ny][nx] codes (wall_code_2d_kernel)
 };
 
 constexpr int kTX = 32, kTY = 16, kWX = kTX + 2, kWY = kTY + 2, kWN = kWX * kWY;
@@ -205,7 +206,29 @@ __device__ __forceinline__ int wrap_mod(int i, int n)
     return r < 0 ? r + n : r;
 }
 
-// The two-step kernel.  a.Uin / a.Uout as in step2d_tile_kernel<false>.
+// The populations of a cell beside internal walls: population q with bits (x, y) of its two-bit code
+// set is replaced by the cell's own one mirrored in x, in y or in both (rho u, rho v negated).
+__device__ __forceinline__ void apply_wall_code(unsigned code, float f[4][4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const unsigned w = code >> (2 * q) & 3u;
+        if (!w) continue;
+#pragma unroll
+        for (int b = 1; b <= 3; ++b) {
+            if (w != (unsigned)b) continue;
+            const int m = b == 1 ? q ^ 1 : (b == 2 ? 3 - q : q ^ 2);
+            f[q][0] = f[m][0];
+            f[q][1] = b & 1 ? -f[m][1] : f[m][1];
+            f[q][2] = b & 2 ? -f[m][2] : f[m][2];
+            f[q][3] = f[m][3];
+        }
+    }
+}
+
+// The two-step kernel.  a.Uin / a.Uout as in step2d_tile_kernel<false>.  WALLS: internal walls, by the
+// cells' codes; solid cells are stepped like others and mean nothing (no fluid cell reads them).
+template <bool WALLS>
 __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
 {
     __shared__ float4 s_f[4 * kAN];      // [q][slot], slot = wy * kAX + wx
@@ -306,6 +329,11 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
             f[q][3] = v.w;
         }
         const int j = j0 + wy;                               // the gathering cell's row (unwrapped)
+        if constexpr (WALLS) {
+            const int ci = wrap_mod(i0 + wx, a.nx), cj = wrap_mod(j, a.ny);
+            const unsigned code = a.walls[LBRS_IX((int64_t)cj * a.nx + ci, a.N, 48)];
+            if (code) apply_wall_code(code, f);
+        }
         const bool wall_bottom = j == 0 && a.bc[2] == BC_WALL;
         const bool wall_top = j == a.ny - 1 && a.bc[3] == BC_WALL;
 #pragma unroll
@@ -359,6 +387,10 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
         f[q][1] = v.y;
         f[q][2] = v.z;
         f[q][3] = v.w;
+    }
+    if constexpr (WALLS) {
+        const unsigned code = a.walls[LBRS_IX((int64_t)j * a.nx + i, a.N, 48)];
+        if (code) apply_wall_code(code, f);
     }
     const bool wall_bottom = j == 0 && a.bc[2] == BC_WALL;
     const bool wall_top = j == a.ny - 1 && a.bc[3] == BC_WALL;
@@ -449,6 +481,7 @@ static F16Args tile_args(const F16StepArgs& s, bool f16)
     a.om1 = s.om1;
     a.c = s.c;
     a.gm1 = s.gm1;
+    a.walls = s.walls;
     return a;
 }
 
@@ -469,7 +502,8 @@ cudaError_t launch_step_f32u(const F16StepArgs& s, cudaStream_t st)
 cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    step2d_u2_kernel<<<grid, kUThreads, 0, st>>>(tile_args(s, false));
+    if (s.walls) step2d_u2_kernel<true><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
+    else step2d_u2_kernel<false><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
     return cudaGetLastError();
 }
 

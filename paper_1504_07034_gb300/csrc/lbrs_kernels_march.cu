@@ -13,7 +13,9 @@ namespace {
 
 constexpr int kSMs = 152, kWarpsPerSM = 16;   // the march's registers allow 16 one-warp blocks per SM
 
-// Moments of the next step's pull from stored distributions: U = sum_q f*_q(x - c_q).
+// Moments of the next step's pull from stored distributions: U = sum_q f*_q(x - c_q).  WALLS: with
+// internal walls (solid cells: the moments of what they hold).
+template <bool WALLS>
 __global__ void __launch_bounds__(256) pull_moments_2d_kernel(const StepArgs<float> a, float* __restrict__ U)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -21,12 +23,23 @@ __global__ void __launch_bounds__(256) pull_moments_2d_kernel(const StepArgs<flo
     if (i >= a.nx || j >= a.ny) return;
     const int64_t c = (int64_t)j * a.nx + i;
     float f[4][4];
-    if (i > 0 && i < a.nx - 1 && j > 0 && j < a.ny - 1) {
-        const int64_t s[4] = {c + a.nx + 1, c + a.nx - 1, c - a.nx - 1, c - a.nx + 1};
+    bool plain = i > 0 && i < a.nx - 1 && j > 0 && j < a.ny - 1;
+    int64_t s[4] = {c + a.nx + 1, c + a.nx - 1, c - a.nx - 1, c - a.nx + 1};
+    if constexpr (WALLS) {
+        if (a.solid[LBRS_IX(c, a.N, 50)]) {
+            plain = true;
+            s[0] = s[1] = s[2] = s[3] = c;
+        } else if (plain) {
+            for (int q = 0; q < 4; ++q) plain &= !a.solid[LBRS_IX(s[q], a.N, 50)];
+        }
+    }
+    if (plain) {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
             for (int k = 0; k < 4; ++k) f[q][k] = a.src[LBRS_IX((q * 4 + k) * a.N + s[q], 16 * a.N, 50)];
+    } else if constexpr (WALLS) {
+        pull_obstacle_2d<float>(a, i, j, f);
     } else {
         pull_edge_2d<float, false>(a, i, j, f);
     }
@@ -36,13 +49,40 @@ __global__ void __launch_bounds__(256) pull_moments_2d_kernel(const StepArgs<flo
             __fadd_rn(__fadd_rn(__fadd_rn(f[0][k], f[1][k]), f[2][k]), f[3][k]);
 }
 
-// f* = f^eq(U) into the populations' planes, two cells a thread.
-__global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restrict__ U, float* __restrict__ f, int64_t N,
-                                                            float c, float gm1)
+// The code of launch_wall_codes, by the rule of pull_obstacle_2d.
+__global__ void __launch_bounds__(256) wall_code_2d_kernel(const StepArgs<float> a, uint8_t* __restrict__ codes)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= a.nx || j >= a.ny) return;
+    const int SX[4] = {-1, 1, 1, -1}, SY[4] = {-1, -1, 1, 1};
+    const int64_t c = (int64_t)j * a.nx + i;
+    unsigned code = 0;
+    if (!a.solid[LBRS_IX(c, a.N, 58)]) {
+        for (int q = 0; q < 4; ++q) {
+            const int si = i - SX[q], sj = j - SY[q];
+            // a wall side's own relation and a Dirichlet ghost go before; solid_at takes both for fluid
+            const bool out_x = si < 0 || si >= a.nx, out_y = sj < 0 || sj >= a.ny;
+            if (out_y && (sj < 0 ? a.bc[2] : a.bc[3]) == BC_WALL) continue;
+            if (out_x && (si < 0 ? a.bc[0] : a.bc[1]) == BC_DIRICHLET) continue;
+            if (!solid_at(a, si, sj)) continue;
+            const bool xn = solid_at(a, si, j), yn = solid_at(a, i, sj);
+            code |= ((yn && !xn ? 0u : 1u) | (xn && !yn ? 0u : 2u)) << (2 * q);
+        }
+    }
+    codes[LBRS_IX(c, a.N, 58)] = (uint8_t)code;
+}
+
+// f* = f^eq(U) into the populations' planes, two cells a thread; solid cells keep theirs.
+__global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restrict__ U, float* __restrict__ f,
+                                                            const uint8_t* __restrict__ solid, int64_t N, float c,
+                                                            float gm1)
 {
     const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= N) return;
-    const bool two = i + 1 < N, vec = (N & 1) == 0;      // vec: every plane starts on 8 bytes
+    const bool two = i + 1 < N;
+    const bool keep0 = solid && solid[i], keep1 = !two || (solid && solid[two ? i + 1 : i]);
+    const bool vec = (N & 1) == 0 && !keep0 && !keep1;   // every plane starts on 8 bytes
     MarchConst m;
     m.c = pk(c, c);
     m.nc = pk(-c, -c);
@@ -55,7 +95,7 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float* p = U + k * N + i;
-        u[k] = vec ? *reinterpret_cast<const P2*>(p) : pk(p[0], two ? p[1] : p[0]);
+        u[k] = pk(p[0], two ? p[1] : p[0]);
     }
     const MarchPrim pr = march_prim(u[0], u[1], u[2], u[3], m);
     auto store = [&](int k) {
@@ -65,8 +105,8 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
             if (vec) {
                 *reinterpret_cast<P2*>(p) = e[q];
             } else {
-                p[0] = lo2(e[q]);
-                if (two) p[1] = hi2(e[q]);
+                if (!keep0) p[0] = lo2(e[q]);
+                if (!keep1) p[1] = hi2(e[q]);
             }
         }
     };
@@ -206,14 +246,23 @@ cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStre
 {
     const dim3 block(64, 4);
     const dim3 grid((unsigned)((a.nx + 63) / 64), (unsigned)((a.ny + 3) / 4));
-    pull_moments_2d_kernel<<<grid, block, 0, s>>>(a, U);
+    if (a.solid) pull_moments_2d_kernel<true><<<grid, block, 0, s>>>(a, U);
+    else pull_moments_2d_kernel<false><<<grid, block, 0, s>>>(a, U);
     return cudaGetLastError();
 }
 
-cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s)
+cudaError_t launch_wall_codes(const StepArgs<float>& a, uint8_t* codes, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((a.nx + 63) / 64), (unsigned)((a.ny + 3) / 4));
+    wall_code_2d_kernel<<<grid, dim3(64, 4), 0, s>>>(a, codes);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_equilibria_f32(const float* U, float* f, const uint8_t* solid, int64_t N, float c, float gm1,
+                                  cudaStream_t s)
 {
     const int64_t threads = (N + 1) / 2;
-    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, N, c, gm1);
+    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, solid, N, c, gm1);
     return cudaGetLastError();
 }
 

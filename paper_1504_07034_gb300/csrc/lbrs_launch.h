@@ -170,7 +170,12 @@ void march_ghosts(const GhostSpec& g, double gamma, double c, float out[4][16]);
 cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaStream_t s);
 // From stored distributions (a.src) the moments U of the next step, and f* = f^eq(U) back.
 cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s);
-cudaError_t launch_equilibria_f32(const float* U, float* f, int64_t N, float c, float gm1, cudaStream_t s);
+// With a mask of solid cells those keep their distributions, and the pull reflects at them (a.solid).
+cudaError_t launch_equilibria_f32(const float* U, float* f, const uint8_t* solid, int64_t N, float c, float gm1,
+                                  cudaStream_t s);
+// Per cell of a grid with internal walls (a.solid), what replaces its populations that are pulled from
+// solid cells: two bits per population, 1 mirrored in x, 2 in y, 3 both; 0 elsewhere.
+cudaError_t launch_wall_codes(const StepArgs<float>& a, uint8_t* codes, cudaStream_t s);
 
 // Scalar D2Q4 in FP32 at omega = 1 on the field u in shared-memory windows (lbrs_scalar.cuh,
 // lbrs_kernels_scalar.cu), bit-identical to single steps; off when LBRS_F32S_WINDOW=0.  Not for
@@ -228,6 +233,7 @@ struct F16StepArgs {
     int nx, ny;
     int bc[4];
     float om, om1, c, gm1;
+    const uint8_t* walls;  // launch_step2_f32u only: the cells' wall codes, or NULL without internal walls
 };
 cudaError_t launch_step_f16neq(const F16StepArgs& a, cudaStream_t s);
 // Moments-only form (omega = 1): a state buffer is U [4][N] FP32.

@@ -284,6 +284,7 @@ F16StepArgs f16_args(const lbrs_ctx* ctx, int from)
     a.om1 = (float)(1.0 - ctx->cfg.omega);
     a.c = (float)ctx->c;
     a.gm1 = (float)(ctx->cfg.gamma - 1.0);
+    a.walls = nullptr;
     return a;
 }
 
@@ -375,15 +376,21 @@ bool fused3(const lbrs_ctx* ctx)
 }
 
 // FP32 at omega = 1 (distributions or moments-only storage) on the moments by the marching kernel
-// (lbrs_march.cuh), two steps a launch?  Not with internal walls (solid cells carry distributions
-// that are no equilibria) or halfway walls; the switches that ask for one, two or three storing
-// steps a launch turn it off as well.
-bool march(const lbrs_ctx* ctx)
+// (lbrs_march.cuh), two steps a launch?  Not with halfway walls; the switches that ask for one, two
+// or three storing steps a launch turn it off as well.  Internal walls step on the moments too, on the
+// tile kernel (a fluid cell never uses what a solid cell holds), but not recording steps.
+bool on_moments(const lbrs_ctx* ctx)
 {
-    if (ctx->f64 || ctx->f16 || ctx->lattice != LBRS_D2Q4 || ctx->cfg.omega != 1.0 || ctx->solid) return false;
+    if (ctx->f64 || ctx->f16 || ctx->lattice != LBRS_D2Q4 || ctx->cfg.omega != 1.0) return false;
     if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
     return march_enabled() && (ctx->f32u ? step2_f32u_enabled() : step2_f32_enabled() && step3_f32_enabled());
 }
+
+bool march(const lbrs_ctx* ctx) { return !ctx->solid && on_moments(ctx); }
+
+// The wall codes of a call on a grid with internal walls, behind the two sets of moments in the
+// idle buffer.
+uint8_t* wall_codes(const lbrs_ctx* ctx) { return (uint8_t*)ctx->f[ctx->cur ^ 1] + 32 * (size_t)ctx->N; }
 
 MarchStep march_step(const lbrs_ctx* ctx, const char* src, char* dst)
 {
@@ -403,10 +410,14 @@ MarchStep march_step(const lbrs_ctx* ctx, const char* src, char* dst)
 // m = 1 or 2 steps on the moments from src into dst.
 cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int m, cudaStream_t s)
 {
-    if (!ctx->mtiles) return launch_march_f32(march_step(ctx, src, dst), m, false, s);
+    if (!ctx->mtiles && !ctx->solid) return launch_march_f32(march_step(ctx, src, dst), m, false, s);
     F16StepArgs a = f16_args(ctx, 0);
     a.src = src;
     a.dst = dst;
+    if (ctx->solid) {
+        if (m != 2) return cudaErrorInvalidValue;
+        a.walls = wall_codes(ctx);
+    }
     return m == 2 ? launch_step2_f32u(a, s) : launch_step_f32u(a, s);
 }
 
@@ -719,7 +730,7 @@ cudaError_t launch_pull_into(lbrs_ctx* ctx, const char* f, char* U)
 cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U)
 {
     ctx->launches += 1;
-    return launch_equilibria_f32((const float*)U, (float*)ctx->f[ctx->cur], ctx->N, (float)ctx->c,
+    return launch_equilibria_f32((const float*)U, (float*)ctx->f[ctx->cur], ctx->solid, ctx->N, (float)ctx->c,
                                  (float)(ctx->cfg.gamma - 1.0), ctx->stream);
 }
 
@@ -1035,11 +1046,22 @@ static bool tube_f64(const lbrs_ctx* ctx)
 // step and leaves through the equilibria of the last, back into the buffer it came from.
 static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
 {
+    int64_t left = n;
+    int launches = 0;
+    if (ctx->solid && (n & 1) == 0) {
+        // with internal walls the moments go two steps at a time: after the pull an even number
+        LBRS_CUDA(ctx, launch_one_step(ctx, ctx->cur, ctx->stream));
+        ctx->cur ^= 1;
+        left -= 1;
+        launches += 1;
+    }
     char* v[2];
     march_buffers(ctx, v);
     const int buf = ctx->f32u ? ctx->cur : ctx->cur ^ 1;
-    int64_t left = n;
-    int launches = 0;
+    if (ctx->solid) {
+        LBRS_CUDA(ctx, launch_wall_codes(step_args<float>(ctx, ctx->cur), wall_codes(ctx), ctx->stream));
+        launches += 1;
+    }
     if (!ctx->f32u) {
         LBRS_CUDA(ctx, launch_pull_moments_f32(step_args<float>(ctx, ctx->cur), (float*)v[0], ctx->stream));
         left -= 1;
@@ -1062,9 +1084,7 @@ static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
     if (ctx->f32u) {
         ctx->cur ^= rest & 1;
     } else {
-        LBRS_CUDA(ctx, launch_equilibria_f32((const float*)v[rest & 1], (float*)ctx->f[ctx->cur], ctx->N, (float)ctx->c,
-                                             (float)(ctx->cfg.gamma - 1.0), ctx->stream));
-        launches += 1;
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, v[rest & 1]));
     }
     ctx->step += n;
     ctx->launches += launches;
@@ -1123,7 +1143,7 @@ static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
     }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBRS_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
-    if (march(ctx) && (ctx->f32u || n >= march_min(ctx))) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
+    if (on_moments(ctx) && (ctx->f32u || n >= march_min(ctx))) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
     int64_t left = n;
     const int G = graph_steps(ctx);
     if (cap == cudaStreamCaptureStatusNone && n >= 2 * G) {
@@ -1302,6 +1322,11 @@ lbrs_status lbrs_set_obstacles(lbrs_ctx* ctx, const uint8_t* d_solid)
         if (ctx->graph[b]) {
             cudaGraphExecDestroy(ctx->graph[b]);
             ctx->graph[b] = nullptr;
+        }
+    for (int b = 0; b < 2; ++b)
+        if (ctx->mgraph[b]) {
+            cudaGraphExecDestroy(ctx->mgraph[b]);
+            ctx->mgraph[b] = nullptr;
         }
     ctx->solid = d_solid;
     return LBRS_OK;

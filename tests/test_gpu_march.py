@@ -62,3 +62,46 @@ def test_march_equals_single_steps(tmp_path):
     assert np.all(np.isfinite(res["single"]))
     for name in ("march", "default"):
         assert np.array_equal(res[name], res["single"]), (name, np.max(np.abs(res[name] - res["single"])))
+
+
+_WALLS_SCRIPT = r"""
+import os
+import sys
+sys.path[:0] = [sys.argv[1], os.path.join(sys.argv[1], "tests")]
+import numpy as np
+import torch
+import workloads as W
+from test_gpu_obstacles import random_obstacle_case
+from paper_1504_07034_gb300.solver import Solver
+cases = [W.forward_facing_step(), W.shock_diffraction(n=100)]
+for k, (nx, ny) in enumerate(((64, 40), (132, 18), (36, 29), (97, 48), (37, 29))):
+    for bcname in ("periodic", "walls_periodic_x", "transmissive", "mixed"):
+        cases.append(random_obstacle_case(nx, ny, bcname, 1.0, seed=7 * k + len(bcname), steps=0))
+out = []
+for wl in cases:
+    s = Solver.from_workload(wl, precision="f32")
+    s.set_state(torch.from_numpy(wl.prim).cuda())
+    for n in (8, 9, 70, 131):                 # even and odd calls, with and without captured graphs
+        s.step(n)
+        out.append(s.get_distributions().cpu().numpy().ravel())
+    s.set_obstacles(None)                     # without walls, and with them again
+    s.step(66)
+    out.append(s.get_distributions().cpu().numpy().ravel())
+    s.set_obstacles(torch.from_numpy(wl.solid))
+    s.step(67)
+    out.append(s.get_distributions().cpu().numpy().ravel())
+    s.close()
+np.save(sys.argv[2], np.concatenate(out))
+"""
+
+
+def test_internal_walls_on_the_moments_equal_single_steps(tmp_path):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    script = tmp_path / "walls.py"
+    script.write_text(_WALLS_SCRIPT)
+    res = {}
+    for name, env in (("moments", {}), ("single", {"LBRS_F32_FUSE": "0"})):
+        out = tmp_path / f"{name}.npy"
+        subprocess.run([sys.executable, str(script), root, str(out)], check=True, env=dict(os.environ, **env), timeout=600)
+        res[name] = np.load(out)
+    assert np.array_equal(res["moments"], res["single"], equal_nan=True)
