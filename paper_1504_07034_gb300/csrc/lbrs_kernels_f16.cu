@@ -226,12 +226,48 @@ __device__ __forceinline__ void apply_wall_code(unsigned code, float f[4][4])
     }
 }
 
-// The two-step kernel.  a.Uin / a.Uout as in step2d_tile_kernel<false>.  WALLS: internal walls, by the
-// cells' codes; solid cells are stepped like others and mean nothing (no fluid cell reads them).
-template <bool WALLS>
-__global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
+// The non-equilibrium parts of populations 0, 1, 2 as the FP16 form stores them: (1 - omega)(f - f^eq)
+// over the field's scale.
+__device__ __forceinline__ __half f16_part(float om1, float f, float e, float inv) { return __float2half_rn(om1 * (f - e) * inv); }
+
+// f* of a slot from its moments and, in the FP16 form, its stored parts (g[q][k / 2]: those of fields
+// k and k + 1).
+template <bool F16>
+__device__ __forceinline__ void rebuild(const F16Args& a, const float U[4], const __half2 (*g)[2], const float sc[4], float e[4][4])
+{
+    equilibria2d<float>(U, a.gm1, a.c, e);
+    if constexpr (F16) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float v[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[q] = k & 1 ? __high2float(g[q][k / 2]) : __low2float(g[q][k / 2]);
+            const float g0 = v[0], g1 = v[1], g2 = v[2];
+            e[0][k] += sc[k] * g0;
+            e[1][k] += sc[k] * g1;
+            e[2][k] += sc[k] * g2;
+            e[3][k] += sc[k] * -((g0 + g1) + g2);
+        }
+    }
+}
+
+// The two-step kernel.  a.Uin / a.Uout as in step2d_tile_kernel.  F16: the FP16 non-equilibrium form,
+// whose parts are rounded to their storage type between the steps as single steps do.  WALLS: internal
+// walls, by the cells' codes; solid cells are stepped like others and mean nothing (no fluid cell reads
+// them).
+template <bool F16, bool WALLS>
+__global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const F16Args a)
 {
     __shared__ float4 s_f[4 * kAN];      // [q][slot], slot = wy * kAX + wx
+    float sc[4] = {1.f, 1.f, 1.f, 1.f}, inv[4] = {1.f, 1.f, 1.f, 1.f};
+    if constexpr (F16) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            sc[k] = a.scale[k];
+            inv[k] = 1.f / sc[k];          // exact: the scales are powers of two
+        }
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) a.scale_out[threadIdx.x] = a.scale[threadIdx.x];
+    }
     const int ti0 = blockIdx.x * kUX, tj0 = blockIdx.y * kUY;
     const int i0 = ti0 - 2, j0 = tj0 - 2;                  // global cell of window slot (0, 0)
     const bool inside = i0 >= 0 && j0 >= 0 && i0 + kAX <= a.nx && j0 + kAY <= a.ny;
@@ -271,8 +307,17 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
         float U[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) U[k] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 43)];
+        __half2 g[3][2];
+        if constexpr (F16) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int k = 0; k < 4; k += 2)
+                    g[q][k / 2] = __halves2half2(a.gin[LBRS_IX((q * 4 + k) * a.N + c, 12 * a.N, 43)],
+                                                 a.gin[LBRS_IX((q * 4 + k + 1) * a.N + c, 12 * a.N, 43)]);
+        }
         float e[4][4];
-        equilibria2d<float>(U, a.gm1, a.c, e);
+        rebuild<F16>(a, U, g, sc, e);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             s_f[LBRS_IX(q * kAN + w, 4 * kAN, 42)] = make_float4(e[q][0], e[q][1], e[q][2], e[q][3]);
@@ -281,6 +326,7 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
 
     // phase B: U^{n+1} of the inner slots (kind 0: skip, 1: gathered, 2: Dirichlet ghost of side gs)
     float U1[kBPer][4];
+    __half2 g1[kBPer][3][2];
     int kind1[kBPer], gs1[kBPer];
 #pragma unroll
     for (int r = 0; r < kBPer; ++r) {
@@ -350,6 +396,16 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) U1[r][k] = ((f[0][k] + f[1][k]) + f[2][k]) + f[3][k];
+        if constexpr (F16) {
+            float e[4][4];
+            equilibria2d<float>(U1[r], a.gm1, a.c, e);
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int k = 0; k < 4; k += 2)
+                    g1[r][q][k / 2] = __halves2half2(f16_part(a.om1, f[q][k], e[q][k], inv[k]),
+                                                     f16_part(a.om1, f[q][k + 1], e[q][k + 1], inv[k + 1]));
+        }
         kind1[r] = 1;
     }
     __syncthreads();
@@ -366,7 +422,7 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
             continue;
         }
         float e[4][4];
-        equilibria2d<float>(U1[r], a.gm1, a.c, e);
+        rebuild<F16>(a, U1[r], g1[r], sc, e);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             s_f[LBRS_IX(q * kAN + w, 4 * kAN, 45)] = make_float4(e[q][0], e[q][1], e[q][2], e[q][3]);
@@ -408,7 +464,21 @@ __global__ void __launch_bounds__(kUThreads) step2d_u2_kernel(const F16Args a)
     }
     const int64_t c = (int64_t)j * a.nx + i;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 47)] = ((f[0][k] + f[1][k]) + f[2][k]) + f[3][k];
+    float U[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        U[k] = ((f[0][k] + f[1][k]) + f[2][k]) + f[3][k];
+        a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 47)] = U[k];
+    }
+    if constexpr (F16) {
+        float e[4][4];
+        equilibria2d<float>(U, a.gm1, a.c, e);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                a.gout[LBRS_IX((q * 4 + k) * a.N + c, 12 * a.N, 47)] = f16_part(a.om1, f[q][k], e[q][k], inv[k]);
+    }
 }
 
 // Initial state: U from W (conserved or primitive, FP64 arithmetic), g = 0.
@@ -502,9 +572,25 @@ cudaError_t launch_step_f32u(const F16StepArgs& s, cudaStream_t st)
 cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    if (s.walls) step2d_u2_kernel<true><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
-    else step2d_u2_kernel<false><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
+    if (s.walls) step2d_u2_kernel<false, true><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
+    else step2d_u2_kernel<false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
     return cudaGetLastError();
+}
+
+cudaError_t launch_step2_f16neq(const F16StepArgs& s, cudaStream_t st)
+{
+    const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
+    step2d_u2_kernel<true, false><<<grid, kUThreads, 0, st>>>(tile_args(s, true));
+    return cudaGetLastError();
+}
+
+bool step2_f16neq_enabled()
+{
+    static const int v = [] {
+        const char* e = getenv("LBRS_F16_FUSE");
+        return (e && !strcmp(e, "0")) ? 0 : 1;
+    }();
+    return v != 0;
 }
 
 bool step2_f32u_enabled()

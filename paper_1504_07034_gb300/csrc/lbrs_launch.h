@@ -236,6 +236,9 @@ struct F16StepArgs {
     const uint8_t* walls;  // launch_step2_f32u only: the cells' wall codes, or NULL without internal walls
 };
 cudaError_t launch_step_f16neq(const F16StepArgs& a, cudaStream_t s);
+// The same, two steps per launch (bit-identical); off when the environment sets LBRS_F16_FUSE=0.
+cudaError_t launch_step2_f16neq(const F16StepArgs& a, cudaStream_t s);
+bool step2_f16neq_enabled();
 // Moments-only form (omega = 1): a state buffer is U [4][N] FP32.
 cudaError_t launch_step_f32u(const F16StepArgs& a, cudaStream_t s);
 // The same, two steps per launch (bit-identical to two single steps); off when the

@@ -361,7 +361,8 @@ bool fused2_scalar(const lbrs_ctx* ctx)
 
 bool fused2(const lbrs_ctx* ctx)
 {
-    return fused2_f32(ctx) || (ctx->f32u && step2_f32u_enabled()) || fused2_scalar(ctx);
+    return fused2_f32(ctx) || (ctx->f32u && step2_f32u_enabled()) || (ctx->f16 && step2_f16neq_enabled()) ||
+           fused2_scalar(ctx);
 }
 
 unsigned* wait_flag(const lbrs_ctx* ctx) { return (unsigned*)(ctx->ws + ctx->L.wait_flag); }
@@ -449,6 +450,7 @@ cudaError_t launch_step3(const lbrs_ctx* ctx, int b, cudaStream_t s)
 cudaError_t launch_step2(const lbrs_ctx* ctx, int b, cudaStream_t s)
 {
     if (ctx->f32u) return launch_step2_f32u(f16_args(ctx, b), s);
+    if (ctx->f16) return launch_step2_f16neq(f16_args(ctx, b), s);
     if (fused2_scalar(ctx)) return launch_step2s_f32(step_args<float>(ctx, b), s);
     return launch_step2_f32(step_args<float>(ctx, b), &ctx->tmap[b], wait_flag(ctx), s);
 }
