@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 
 #include "lbrs_kernels.cuh"
+#include "lbrs_adapt.cuh"
 #include "lbrs_launch.h"
 
 namespace lbrs {
@@ -197,6 +198,48 @@ constexpr int kBX = kUX + 2, kBY = kUY + 2, kBN = kBX * kBY;   // phase-B inner 
 constexpr int kUThreads = kUX * kUY;
 constexpr int kBPer = (kBN + kUThreads - 1) / kUThreads;       // inner slots per thread
 
+// The wall sides' populations of a cell of row j from its own, mirrored.
+__device__ __forceinline__ void wall_relations(const F16Args& a, int j, float f[4][4])
+{
+    const bool wall_bottom = j == 0 && a.bc[2] == BC_WALL;
+    const bool wall_top = j == a.ny - 1 && a.bc[3] == BC_WALL;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float sgn = k == 2 ? -1.f : 1.f;
+        if (wall_top) {
+            f[0][k] = sgn * f[3][k];
+            f[1][k] = sgn * f[2][k];
+        }
+        if (wall_bottom) {
+            f[3][k] = sgn * f[0][k];
+            f[2][k] = sgn * f[1][k];
+        }
+    }
+}
+
+// The inner slots of a thread: its own cell's, then (the last threads, as phase A's second round falls to
+// the first) one of the frame's, so that the tile's own cells are one round of full warps.  The FP16 form
+// takes them row by row (this order costs it 5% in registers kept on the stack).
+static_assert(kUThreads + 2 * (kBX + kUY) == kBN && kBPer == 2, "inner slots: the tile's cells and a frame");
+__device__ __forceinline__ bool inner_slot(int r, int& wx, int& wy)
+{
+    const int t = r == 0 ? threadIdx.x : kUThreads - 1 - threadIdx.x;
+    if (r == 0) {
+        wx = 2 + t % kUX;
+        wy = 2 + t / kUX;
+        return true;
+    }
+    const int e = t - 2 * kBX;
+    wx = 1 + (e < 0 ? (t < kBX ? t : t - kBX) : (e < kUY ? 0 : kBX - 1));
+    wy = 1 + (e < 0 ? (t < kBX ? 0 : kBY - 1) : 1 + (e < kUY ? e : e - kUY));
+    return e < 2 * kUY;
+}
+
+__device__ __forceinline__ void add_bound(unsigned bits, unsigned long long* dst)
+{
+    if (bits) atomicMax(dst, (unsigned long long)__double_as_longlong((double)__uint_as_float(bits)));
+}
+
 // Cells beyond side s of an axis of n cells that a coordinate lies (0 inside).
 __device__ __forceinline__ int beyond(int i, int n) { return i < 0 ? -i : (i >= n ? i - n + 1 : 0); }
 
@@ -233,9 +276,10 @@ __device__ __forceinline__ __half f16_part(float om1, float f, float e, float in
 // f* of a slot from its moments and, in the FP16 form, its stored parts (g[q][k / 2]: those of fields
 // k and k + 1).
 template <bool F16>
-__device__ __forceinline__ void rebuild(const F16Args& a, const float U[4], const __half2 (*g)[2], const float sc[4], float e[4][4])
+__device__ __forceinline__ void rebuild(const F16Args& a, float c, const float U[4], const __half2 (*g)[2],
+                                        const float sc[4], float e[4][4])
 {
-    equilibria2d<float>(U, a.gm1, a.c, e);
+    equilibria2d<float>(U, a.gm1, c, e);
     if constexpr (F16) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -254,9 +298,11 @@ __device__ __forceinline__ void rebuild(const F16Args& a, const float U[4], cons
 // The two-step kernel.  a.Uin / a.Uout as in step2d_tile_kernel.  F16: the FP16 non-equilibrium form,
 // whose parts are rounded to their storage type between the steps as single steps do.  WALLS: internal
 // walls, by the cells' codes; solid cells are stepped like others and mean nothing (no fluid cell reads
-// them).
-template <bool F16, bool WALLS>
-__global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const F16Args a)
+// them).  ADAPT: adaptive lambda (lbrs_adapt.cuh; no Dirichlet sides), the bounds of both new states.  Every
+// block takes the clock forward while its loads are under way: 4 of a launch's 19 us at 768 x 768 (the
+// bounds 2 us), against a launch of its own or a last block's turn at about as much.
+template <bool F16, bool WALLS, bool ADAPT>
+__global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const F16Args a, const AdaptPair ad)
 {
     __shared__ float4 s_f[4 * kAN];      // [q][slot], slot = wy * kAX + wx
     float sc[4] = {1.f, 1.f, 1.f, 1.f}, inv[4] = {1.f, 1.f, 1.f, 1.f};
@@ -272,7 +318,69 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     const int i0 = ti0 - 2, j0 = tj0 - 2;                  // global cell of window slot (0, 0)
     const bool inside = i0 >= 0 && j0 >= 0 && i0 + kAX <= a.nx && j0 + kAY <= a.ny;
     const bool per_x = a.bc[0] == BC_PERIODIC, per_y = a.bc[2] == BC_PERIODIC;
-
+    float c0 = a.c, c1 = a.c;
+    __shared__ unsigned s_max[2];                          // ADAPT: largest bounds of the tile's new states
+    const float g32 = (float)ad.gamma;
+    const unsigned slot8 = (blockIdx.x + blockIdx.y * gridDim.x) % kBoundSlots;
+    bool skip2 = false;                                    // the second step lies beyond the run's end
+    if constexpr (ADAPT) {
+        // phase A, its loads under way while the first warp takes the clock forward
+        if (threadIdx.x < 2) s_max[threadIdx.x] = 0u;
+        __shared__ float s_c[2];
+        __shared__ int s_skip[2];
+        constexpr int kAPer = (kAN + kUThreads - 1) / kUThreads;
+        float Ua[kAPer][4];
+        bool any[kAPer];
+#pragma unroll
+        for (int r = 0; r < kAPer; ++r) {
+            const int w = threadIdx.x + r * kUThreads;
+            int i = i0 + w % kAX, j = j0 + w / kAX;
+            any[r] = w < kAN;
+            if (!inside) {
+                const int bx = beyond(i, a.nx), by = beyond(j, a.ny);
+                if ((bx > 1 && !per_x) || (by > 1 && !per_y) || bx > 2 || by > 2) any[r] = false;
+                if (bx) i = per_x ? wrap_mod(i, a.nx) : (i < 0 ? 0 : a.nx - 1);
+                if (by) j = per_y ? wrap_mod(j, a.ny) : (j < 0 ? 0 : a.ny - 1);
+            }
+            const int64_t c = (int64_t)j * a.nx + i;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) Ua[r][k] = any[r] ? a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 47)] : 1.f;
+        }
+        if (threadIdx.x < 32) {
+            AdaptRun r1, r2;
+            adapt_clocks(*ad.in, ad.bounds_in, ad.pending, ad.dx, ad.safety, ad.t_final, r1, r2);
+            if (threadIdx.x == 0) {
+                s_c[0] = (float)r1.c;
+                s_skip[0] = r1.done;
+                s_c[1] = (float)r2.c;
+                s_skip[1] = r2.done;
+                if (blockIdx.x == 0 && blockIdx.y == 0) *ad.out = r2;
+            }
+            if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2 * kBoundSlots) ad.bounds_clear[threadIdx.x] = 0ull;
+        }
+        __syncthreads();
+        c0 = s_c[0];
+        c1 = s_c[1];
+        skip2 = s_skip[1];
+        if (s_skip[0]) {                                   // both: the state stays
+            const int i = ti0 + (int)threadIdx.x % kUX, j = tj0 + (int)threadIdx.x / kUX;
+            if (i >= a.nx || j >= a.ny) return;
+            const int64_t c = (int64_t)j * a.nx + i;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 59)];
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < kAPer; ++r) {
+            const int w = threadIdx.x + r * kUThreads;
+            if (!any[r]) continue;
+            float e[4][4];
+            equilibria2d<float>(Ua[r], a.gm1, c0, e);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                s_f[LBRS_IX(q * kAN + w, 4 * kAN, 46)] = make_float4(e[q][0], e[q][1], e[q][2], e[q][3]);
+        }
+    } else
     // phase A: f*^n of every window slot that a later phase reads
     for (int w = threadIdx.x; w < kAN; w += kUThreads) {
         int i = i0 + w % kAX, j = j0 + w / kAX;
@@ -317,7 +425,7 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
                                                  a.gin[LBRS_IX((q * 4 + k + 1) * a.N + c, 12 * a.N, 43)]);
         }
         float e[4][4];
-        rebuild<F16>(a, U, g, sc, e);
+        rebuild<F16>(a, c0, U, g, sc, e);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             s_f[LBRS_IX(q * kAN + w, 4 * kAN, 42)] = make_float4(e[q][0], e[q][1], e[q][2], e[q][3]);
@@ -332,9 +440,15 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     for (int r = 0; r < kBPer; ++r) {
         kind1[r] = 0;
         gs1[r] = 0;
-        const int b = threadIdx.x + r * kUThreads;
-        if (b >= kBN) continue;
-        int wx = 1 + b % kBX, wy = 1 + b / kBX;             // window position of the slot
+        int wx, wy;                                          // window position of the slot
+        if constexpr (F16) {
+            const int b = threadIdx.x + r * kUThreads;
+            if (b >= kBN) continue;
+            wx = 1 + b % kBX;
+            wy = 1 + b / kBX;
+        } else {
+            if (!inner_slot(r, wx, wy)) continue;
+        }
         if (!inside) {
             const int i = i0 + wx, j = j0 + wy;
             const int bx = beyond(i, a.nx), by = beyond(j, a.ny);
@@ -380,20 +494,7 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
             const unsigned code = a.walls[LBRS_IX((int64_t)cj * a.nx + ci, a.N, 48)];
             if (code) apply_wall_code(code, f);
         }
-        const bool wall_bottom = j == 0 && a.bc[2] == BC_WALL;
-        const bool wall_top = j == a.ny - 1 && a.bc[3] == BC_WALL;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float sgn = k == 2 ? -1.f : 1.f;
-            if (wall_top) {
-                f[0][k] = sgn * f[3][k];
-                f[1][k] = sgn * f[2][k];
-            }
-            if (wall_bottom) {
-                f[3][k] = sgn * f[0][k];
-                f[2][k] = sgn * f[1][k];
-            }
-        }
+        if (F16 || !inside) wall_relations(a, j, f);
 #pragma unroll
         for (int k = 0; k < 4; ++k) U1[r][k] = ((f[0][k] + f[1][k]) + f[2][k]) + f[3][k];
         if constexpr (F16) {
@@ -408,12 +509,34 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
         }
         kind1[r] = 1;
     }
+    if constexpr (ADAPT) {
+        const int i = ti0 + (int)threadIdx.x % kUX, j = tj0 + (int)threadIdx.x / kUX;   // inner_slot(0)
+        const bool in = i < a.nx && j < a.ny;
+        const unsigned m = __reduce_max_sync(0xffffffffu, in ? bound_bits(U1[0], g32, a.gm1) : 0u);
+        if (threadIdx.x % 32 == 0) atomicMax(&s_max[0], m);
+        if (skip2 && in) {
+            const int64_t c = (int64_t)j * a.nx + i;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = U1[0][k];
+        }
+    }
     __syncthreads();
+    if constexpr (ADAPT) {
+        if (threadIdx.x == 0) add_bound(s_max[0], ad.bounds_out + slot8);
+        if (skip2) return;
+    }
 #pragma unroll
     for (int r = 0; r < kBPer; ++r) {
-        const int b = threadIdx.x + r * kUThreads;
-        if (b >= kBN || kind1[r] == 0) continue;
-        const int w = (1 + b / kBX) * kAX + 1 + b % kBX;
+        int wx, wy;
+        if constexpr (F16) {
+            const int b = threadIdx.x + r * kUThreads;
+            if (b >= kBN || kind1[r] == 0) continue;
+            wx = 1 + b % kBX;
+            wy = 1 + b / kBX;
+        } else {
+            if (!inner_slot(r, wx, wy) || kind1[r] == 0) continue;
+        }
+        const int w = wy * kAX + wx;
         if (kind1[r] == 2) {
             const float* g = a.ghost + gs1[r] * GHOST_STRIDE;
 #pragma unroll
@@ -422,7 +545,7 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
             continue;
         }
         float e[4][4];
-        rebuild<F16>(a, U1[r], g1[r], sc, e);
+        rebuild<F16>(a, c1, U1[r], g1[r], sc, e);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             s_f[LBRS_IX(q * kAN + w, 4 * kAN, 45)] = make_float4(e[q][0], e[q][1], e[q][2], e[q][3]);
@@ -432,7 +555,8 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     // phase C: U^{n+2} of the tile
     const int tx = threadIdx.x % kUX, ty = threadIdx.x / kUX;
     const int i = ti0 + tx, j = tj0 + ty;
-    if (i >= a.nx || j >= a.ny) return;
+    if (!ADAPT && (i >= a.nx || j >= a.ny)) return;
+    const bool in_grid = i < a.nx && j < a.ny;
     const int slot = (ty + 2) * kAX + (tx + 2);
     const int src[4] = {slot + kAX + 1, slot + kAX - 1, slot - kAX - 1, slot - kAX + 1};
     float f[4][4];
@@ -448,27 +572,20 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
         const unsigned code = a.walls[LBRS_IX((int64_t)j * a.nx + i, a.N, 48)];
         if (code) apply_wall_code(code, f);
     }
-    const bool wall_bottom = j == 0 && a.bc[2] == BC_WALL;
-    const bool wall_top = j == a.ny - 1 && a.bc[3] == BC_WALL;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float sgn = k == 2 ? -1.f : 1.f;
-        if (wall_top) {
-            f[0][k] = sgn * f[3][k];
-            f[1][k] = sgn * f[2][k];
-        }
-        if (wall_bottom) {
-            f[3][k] = sgn * f[0][k];
-            f[2][k] = sgn * f[1][k];
-        }
-    }
+    if (F16 || !inside) wall_relations(a, j, f);
     const int64_t c = (int64_t)j * a.nx + i;
 #pragma unroll
     float U[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         U[k] = ((f[0][k] + f[1][k]) + f[2][k]) + f[3][k];
-        a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 47)] = U[k];
+        if (!ADAPT || in_grid) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 47)] = U[k];
+    }
+    if constexpr (ADAPT) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, in_grid ? bound_bits(U, g32, a.gm1) : 0u);
+        if (threadIdx.x % 32 == 0) atomicMax(&s_max[1], m);
+        __syncthreads();
+        if (threadIdx.x == 0) add_bound(s_max[1], ad.bounds_out + kBoundSlots + slot8);
     }
     if constexpr (F16) {
         float e[4][4];
@@ -572,15 +689,22 @@ cudaError_t launch_step_f32u(const F16StepArgs& s, cudaStream_t st)
 cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    if (s.walls) step2d_u2_kernel<false, true><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
-    else step2d_u2_kernel<false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false));
+    if (s.walls) step2d_u2_kernel<false, true, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false), AdaptPair{});
+    else step2d_u2_kernel<false, false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false), AdaptPair{});
     return cudaGetLastError();
 }
 
 cudaError_t launch_step2_f16neq(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    step2d_u2_kernel<true, false><<<grid, kUThreads, 0, st>>>(tile_args(s, true));
+    step2d_u2_kernel<true, false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, true), AdaptPair{});
+    return cudaGetLastError();
+}
+
+cudaError_t launch_step2_adapt_f32(const F16StepArgs& s, const AdaptPair& ad, cudaStream_t st)
+{
+    const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
+    step2d_u2_kernel<false, false, true><<<grid, kUThreads, 0, st>>>(tile_args(s, false), ad);
     return cudaGetLastError();
 }
 

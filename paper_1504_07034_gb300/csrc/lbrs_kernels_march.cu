@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include "lbrs_adapt.cuh"
 #include "lbrs_march.cuh"
 #include "lbrs_launch.h"
 
@@ -73,11 +74,71 @@ __global__ void __launch_bounds__(256) wall_code_2d_kernel(const StepArgs<float>
     codes[LBRS_IX(c, a.N, 58)] = (uint8_t)code;
 }
 
-// f* = f^eq(U) into the populations' planes, two cells a thread; solid cells keep theirs.
+// An adaptive step's moments and their bound (adapt_prep_kernel has run).
+__global__ void __launch_bounds__(256) adapt_pull_kernel(const StepArgs<float> a, float* __restrict__ U, AdaptState* st,
+                                                         double gamma)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    float bnd = -1.f;
+    if (i < a.nx && j < a.ny) {
+        const int64_t c = (int64_t)j * a.nx + i;
+        float f[4][4], u[4];
+        pull_edge_2d<float, false>(a, i, j, f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            u[k] = __fadd_rn(__fadd_rn(__fadd_rn(f[0][k], f[1][k]), f[2][k]), f[3][k]);
+            U[LBRS_IX(k * a.N + c, 4 * a.N, 60)] = u[k];
+        }
+        bnd = bound_local<float>(u, gamma);
+    }
+    block_max_into<256>(bnd, &st->bound_bits[st->slot_cur]);
+}
+
+__global__ void adapt_enter_kernel(const AdaptState* st, AdaptRun* run, unsigned long long* bounds, double dx)
+{
+    for (int n = threadIdx.x; n < 6 * kBoundSlots; n += 32)
+        bounds[n] = n == kBoundSlots ? st->bound_bits[st->slot_cur] : 0ull;
+    if (threadIdx.x != 0) return;
+    run->t = st->t;
+    run->lam = st->lam_cur;
+    run->c = st->c_new;
+    run->dt = __ddiv_rn(dx, st->lam_cur);
+    run->steps = st->steps;
+    run->last = st->last;
+    run->done = st->done;
+    run->dead = st->skip;
+}
+
+__global__ void adapt_leave_kernel(AdaptState* st, AdaptRun* run, const unsigned long long* last, double dx,
+                                   double safety, double t_final)
+{
+    AdaptRun r, unused;
+    adapt_clocks(*run, last, 2, dx, safety, t_final, r, unused);     // the last state's own clock step
+    if (threadIdx.x != 0) return;
+    unsigned long long b = 0ull;
+    for (int n = 0; n < kBoundSlots; ++n) b = last[kBoundSlots + n] > b ? last[kBoundSlots + n] : b;
+    *run = r;
+    st->t = r.t;
+    st->lam_cur = r.lam;
+    st->c_new = r.c;
+    st->steps = r.steps;
+    st->last = r.last;
+    st->done = r.done;
+    st->bound_bits[st->slot_cur] = b;
+}
+
+// f* = f^eq(U) into the populations' planes, two cells a thread; solid cells keep theirs.  run: the
+// adaptive record whose lambda the distributions take (nothing is written if its run had ended).
 __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restrict__ U, float* __restrict__ f,
-                                                            const uint8_t* __restrict__ solid, int64_t N, float c,
+                                                            const uint8_t* __restrict__ solid,
+                                                            const AdaptRun* __restrict__ run, int64_t N, float c,
                                                             float gm1)
 {
+    if (run) {
+        if (run->dead) return;
+        c = (float)run->c;
+    }
     const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= N) return;
     const bool two = i + 1 < N;
@@ -262,7 +323,39 @@ cudaError_t launch_equilibria_f32(const float* U, float* f, const uint8_t* solid
                                   cudaStream_t s)
 {
     const int64_t threads = (N + 1) / 2;
-    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, solid, N, c, gm1);
+    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, solid, nullptr, N, c, gm1);
+    return cudaGetLastError();
+}
+
+bool adapt_moments_enabled()
+{
+    static const int v = [] {
+        const char* e = getenv("LBRS_F32_ADAPT_MOMENTS");
+        return (e && !strcmp(e, "0")) ? 0 : 1;
+    }();
+    return v != 0;
+}
+
+cudaError_t launch_adapt_enter_f32(const StepArgs<float>& a, float* U, void* st, void* run0,
+                                   unsigned long long* bounds, double gamma, double dx, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((a.nx + 63) / 64), (unsigned)((a.ny + 3) / 4));
+    adapt_pull_kernel<<<grid, dim3(64, 4), 0, s>>>(a, U, (AdaptState*)st, gamma);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    adapt_enter_kernel<<<1, 32, 0, s>>>((const AdaptState*)st, (AdaptRun*)run0, bounds, dx);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adapt_leave_f32(const float* U, float* f, int64_t N, float gm1, void* st, void* run,
+                                   const unsigned long long* last_bounds, double dx, double safety, double t_final,
+                                   cudaStream_t s)
+{
+    adapt_leave_kernel<<<1, 32, 0, s>>>((AdaptState*)st, (AdaptRun*)run, last_bounds, dx, safety, t_final);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int64_t threads = (N + 1) / 2;
+    equilibria_2d_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(U, f, nullptr, (const AdaptRun*)run, N, 0.f, gm1);
     return cudaGetLastError();
 }
 

@@ -245,6 +245,19 @@ cudaError_t launch_step_f32u(const F16StepArgs& a, cudaStream_t s);
 // environment sets LBRS_F32U_FUSE=0.
 cudaError_t launch_step2_f32u(const F16StepArgs& a, cudaStream_t s);
 bool step2_f32u_enabled();
+// Two adaptive steps at omega = 1 on the moments (lbrs_adapt.cuh), sides without Dirichlet states.
+struct AdaptPair;
+cudaError_t launch_step2_adapt_f32(const F16StepArgs& a, const AdaptPair& ad, cudaStream_t s);
+// Into such a chain: the step that adapt_prep_kernel has set up, from the distributions a.src to its
+// moments U and their bound; st the AdaptState, run0 the chain's record, bounds its three pairs.  Out of
+// it: the state from the record `run` after the clock's last step, and the distributions (kept if the run
+// had ended before).  LBRS_F32_ADAPT_MOMENTS=0 turns the chains off.
+cudaError_t launch_adapt_enter_f32(const StepArgs<float>& a, float* U, void* st, void* run0,
+                                   unsigned long long* bounds, double gamma, double dx, cudaStream_t s);
+cudaError_t launch_adapt_leave_f32(const float* U, float* f, int64_t N, float gm1, void* st, void* run,
+                                   const unsigned long long* last_bounds, double dx, double safety, double t_final,
+                                   cudaStream_t s);
+bool adapt_moments_enabled();
 cudaError_t launch_set_state_f32u(const void* W, int w_dtype, int kind, void* fs, int64_t N, int64_t plane,
                                   double gamma, cudaStream_t s);
 // U = U(W) in FP32, g = 0, then the per-field scales from max |U_k| (absmax_bits: 4 words of scratch).

@@ -17,6 +17,7 @@
 
 #include "lbrs.h"
 #include "lbrs_kernels.cuh"
+#include "lbrs_adapt.cuh"
 #include "lbrs_batch.cuh"
 #include "lbrs_launch.h"
 
@@ -35,7 +36,8 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // store_bytes: one stored buffer, which also holds the ghost rows of cut sides;
 // each of the two buffers takes a slot that can also stage K FP64 fields of host input.
 struct Layout {
-    size_t f_bytes, store_bytes, slot, f0, f1, ghost, partials, diag_out, scale, status, wait_flag, adapt, total;
+    size_t f_bytes, store_bytes, slot, f0, f1, ghost, partials, diag_out, scale, status, wait_flag, adapt, adapt_run,
+        total;
 };
 
 bool two_d(int lat) { return lat == LBRS_D2Q4 || lat == LBRS_D2Q4S; }
@@ -97,6 +99,8 @@ Layout layout_of(const lbrs_config* c)
     off += align_up(sizeof(unsigned));
     L.adapt = off;                                   // the adaptive-lambda run's record
     off += align_up(sizeof(AdaptState));
+    L.adapt_run = off;                               // records and bounds of its chains on the moments
+    off += align_up(2 * sizeof(AdaptRun) + 6 * kBoundSlots * sizeof(unsigned long long));
     L.total = off;
     return L;
 }
@@ -1384,6 +1388,19 @@ static lbrs_status ensure_adapt_graph(lbrs_ctx* ctx, int from, double safety, do
     return LBRS_OK;
 }
 
+// FP32 at omega = 1 on the moments, two adaptive steps a launch?  Not beside Dirichlet sides (their
+// ghosts change with lambda) or halfway walls.  From calls of 8 steps on, where entering and leaving the
+// chain has paid on every grid (us per step, chain against storing steps: 64^2 calls of 8 steps 7.3
+// against 9.8, of 256 4.2 against 5.5; 400^2 8.6 against 13.9, 5.2 against 9.0; 1200^2 28 against 41,
+// 19.7 against 35.7).
+static bool adapt_on_moments(const lbrs_ctx* ctx)
+{
+    if (!march(ctx) || ctx->f32u || !adapt_moments_enabled()) return false;
+    for (int s = 0; s < 4; ++s)
+        if (ctx->cfg.bc[s].kind == LBRS_BC_DIRICHLET) return false;
+    return true;
+}
+
 lbrs_status lbrs_step_adaptive(lbrs_ctx* ctx, int64_t n, double safety, double t_final)
 {
     NvtxRange range("lbrs_step_adaptive");
@@ -1410,6 +1427,48 @@ lbrs_status lbrs_step_adaptive(lbrs_ctx* ctx, int64_t n, double safety, double t
     }
     ctx->adapt_used = true;
     int64_t left = n;
+    if (adapt_on_moments(ctx) && n >= 8) {
+        // an odd step first: after the one that enters the chain its steps go in pairs
+        if ((n & 1) == 0) {
+            LBRS_CUDA(ctx, launch_adapt_pair(ctx, ctx->cur, safety, t_final, ctx->stream));
+            ctx->cur ^= 1;
+            ctx->launches += 2;
+            left -= 1;
+        }
+        char* v[2];
+        march_buffers(ctx, v);
+        AdaptRun* run = (AdaptRun*)(ctx->ws + ctx->L.adapt_run);
+        unsigned long long* bounds = (unsigned long long*)(run + 2);      // three pairs of states taking turns
+        LBRS_CUDA(ctx, launch_adapt_prep(0, st, ctx->ws + ctx->L.ghost, ctx->gspec, ctx->cfg.gamma, ctx->cfg.dx, safety,
+                                         t_final, ctx->stream));
+        LBRS_CUDA(ctx, launch_adapt_enter_f32(step_args<float>(ctx, ctx->cur), (float*)v[0], st, run, bounds,
+                                              ctx->cfg.gamma, ctx->cfg.dx, ctx->stream));
+        left -= 1;
+        int j = 0;
+        for (; left > 0; left -= 2, ++j) {
+            F16StepArgs a = f16_args(ctx, 0);
+            a.src = v[j & 1];
+            a.dst = v[(j & 1) ^ 1];
+            AdaptPair p;
+            p.in = run + (j & 1);
+            p.out = run + ((j & 1) ^ 1);
+            p.bounds_in = bounds + 2 * kBoundSlots * (j % 3);
+            p.bounds_out = bounds + 2 * kBoundSlots * ((j + 1) % 3);
+            p.bounds_clear = bounds + 2 * kBoundSlots * ((j + 2) % 3);
+            p.pending = j ? 2 : 1;
+            p.dx = ctx->cfg.dx;
+            p.safety = safety;
+            p.t_final = t_final;
+            p.gamma = ctx->cfg.gamma;
+            LBRS_CUDA(ctx, launch_step2_adapt_f32(a, p, ctx->stream));
+        }
+        LBRS_CUDA(ctx, launch_adapt_leave_f32((const float*)v[j & 1], (float*)ctx->f[ctx->cur], ctx->N,
+                                              (float)(ctx->cfg.gamma - 1.0), st, run + (j & 1), bounds + 2 * kBoundSlots * (j % 3),
+                                              ctx->cfg.dx, safety, t_final, ctx->stream));
+        ctx->launches += 5 + j;
+        ctx->step += n;
+        return LBRS_OK;
+    }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBRS_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
     if (cap == cudaStreamCaptureStatusNone && n >= kAdaptGraphSteps) {
