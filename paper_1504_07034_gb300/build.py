@@ -1,12 +1,13 @@
 """Build the LBRS CUDA library (liblbrs.so) in-tree for sm_103a.
 
-Nine translation units compiled in parallel with nvcc, then linked into one
+Ten translation units compiled in parallel with nvcc, then linked into one
 shared library with the CUDA runtime linked statically:
 
   csrc/lbrs_kernels_f64.cu  FP64 kernels, -fmad=false (rounding as written)
   csrc/lbrs_kernels_f32.cu  FP32 step kernels
   csrc/lbrs_kernels_f16.cu  D2Q4 step with FP16 non-equilibrium storage
   csrc/lbrs_kernels_march.cu FP32 D2Q4 steps at omega = 1 on the moments
+  csrc/lbrs_kernels_fmarch.cu FP32 D2Q4 steps at omega != 1, two a launch in registers
   csrc/lbrs_kernels_tube.cu FP32 1-D tubes in registers
   csrc/lbrs_kernels_scalar.cu FP32 scalar D2Q4 steps in shared-memory windows
   csrc/lbrs_runtime.cu      host C ABI (include/lbrs.h)
@@ -44,6 +45,7 @@ UNITS = {
     "lbrs_kernels_f64.cu": ["-fmad=false"],
     "lbrs_kernels_f32.cu": [],
     "lbrs_kernels_f16.cu": [],
+    "lbrs_kernels_fmarch.cu": [],
     "lbrs_kernels_march.cu": [],
     "lbrs_kernels_tube.cu": [],
     "lbrs_kernels_scalar.cu": [],

@@ -258,6 +258,11 @@ cudaError_t launch_adapt_leave_f32(const float* U, float* f, int64_t N, float gm
                                    const unsigned long long* last_bounds, double dx, double safety, double t_final,
                                    cudaStream_t s);
 bool adapt_moments_enabled();
+// FP32 distribution form, omega != 1: two steps per launch, marching (lbrs_kernels_fmarch.cu); a.Uout: both
+// steps' moments.  No internal walls, no halfway walls.  LBRS_F32_FMARCH=0 turns it off.
+cudaError_t launch_fmarch_f32(const StepArgs<float>& a, const float ghost[4][GHOST_STRIDE], cudaStream_t s);
+bool fmarch_enabled();
+bool fmarch_beats_tiles(int nx, int ny);
 cudaError_t launch_set_state_f32u(const void* W, int w_dtype, int kind, void* fs, int64_t N, int64_t plane,
                                   double gamma, cudaStream_t s);
 // U = U(W) in FP32, g = 0, then the per-field scales from max |U_k| (absmax_bits: 4 words of scratch).

@@ -373,12 +373,23 @@ unsigned* wait_flag(const lbrs_ctx* ctx) { return (unsigned*)(ctx->ws + ctx->L.w
 
 // The FP32 three-steps-per-launch kernel available for this context?  Not with internal
 // walls or halfway walls (their populations break the one-reader rule of its in-place phases).
-bool fused3(const lbrs_ctx* ctx)
+bool step3_tiles(const lbrs_ctx* ctx)
 {
     if (!fused2_f32(ctx) || ctx->solid || !step3_f32_enabled()) return false;
     if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
     return ctx->tmap3[0].valid && ctx->tmap3[1].valid;
 }
+
+// FP32 distributions at omega != 1 two steps a launch by the marching kernel (lbrs_kernels_fmarch.cu)?
+// The switches that ask for one or two storing steps a launch turn it off.
+bool fmarch(const lbrs_ctx* ctx)
+{
+    if (!fmarch_enabled() || !fused2_f32(ctx) || !step3_f32_enabled() || ctx->solid || ctx->cfg.omega == 1.0) return false;
+    if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
+    return !step3_tiles(ctx) || fmarch_beats_tiles((int)ctx->cfg.nx, (int)ctx->ny_store);
+}
+
+bool fused3(const lbrs_ctx* ctx) { return step3_tiles(ctx) && !fmarch(ctx); }
 
 // FP32 at omega = 1 (distributions or moments-only storage) on the moments by the marching kernel
 // (lbrs_march.cuh), two steps a launch?  Not with halfway walls; the switches that ask for one, two
@@ -456,6 +467,7 @@ cudaError_t launch_step2(const lbrs_ctx* ctx, int b, cudaStream_t s)
     if (ctx->f32u) return launch_step2_f32u(f16_args(ctx, b), s);
     if (ctx->f16) return launch_step2_f16neq(f16_args(ctx, b), s);
     if (fused2_scalar(ctx)) return launch_step2s_f32(step_args<float>(ctx, b), s);
+    if (fmarch(ctx)) return launch_fmarch_f32(step_args<float>(ctx, b), ctx->mghost, s);
     return launch_step2_f32(step_args<float>(ctx, b), &ctx->tmap[b], wait_flag(ctx), s);
 }
 
@@ -698,6 +710,7 @@ cudaError_t launch_record_step2(lbrs_ctx* ctx, void* Uout)
 {
     StepArgs<float> a = step_args<float>(ctx, ctx->cur);
     a.Uout = (float*)Uout;
+    if (fmarch(ctx)) return launch_fmarch_f32(a, ctx->mghost, ctx->stream);
     return launch_step2_f32(a, &ctx->tmap[ctx->cur], wait_flag(ctx), ctx->stream);
 }
 
