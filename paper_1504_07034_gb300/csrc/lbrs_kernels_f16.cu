@@ -29,6 +29,7 @@
 
 #include <cuda_fp16.h>
 
+#include "lbrs_chain.cuh"
 #include "lbrs_kernels.cuh"
 #include "lbrs_adapt.cuh"
 #include "lbrs_launch.h"
@@ -305,6 +306,7 @@ template <bool F16, bool WALLS, bool ADAPT>
 __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const F16Args a, const AdaptPair ad)
 {
     __shared__ float4 s_f[4 * kAN];      // [q][slot], slot = wy * kAX + wx
+    chain_begin();
     float sc[4] = {1.f, 1.f, 1.f, 1.f}, inv[4] = {1.f, 1.f, 1.f, 1.f};
     if constexpr (F16) {
 #pragma unroll
@@ -689,23 +691,21 @@ cudaError_t launch_step_f32u(const F16StepArgs& s, cudaStream_t st)
 cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    if (s.walls) step2d_u2_kernel<false, true, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false), AdaptPair{});
-    else step2d_u2_kernel<false, false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, false), AdaptPair{});
-    return cudaGetLastError();
+    if (s.walls)
+        return launch_in_chain(s.chained, step2d_u2_kernel<false, true, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
+    return launch_in_chain(s.chained, step2d_u2_kernel<false, false, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
 }
 
 cudaError_t launch_step2_f16neq(const F16StepArgs& s, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    step2d_u2_kernel<true, false, false><<<grid, kUThreads, 0, st>>>(tile_args(s, true), AdaptPair{});
-    return cudaGetLastError();
+    return launch_in_chain(s.chained, step2d_u2_kernel<true, false, false>, grid, kUThreads, st, tile_args(s, true), AdaptPair{});
 }
 
 cudaError_t launch_step2_adapt_f32(const F16StepArgs& s, const AdaptPair& ad, cudaStream_t st)
 {
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
-    step2d_u2_kernel<false, false, true><<<grid, kUThreads, 0, st>>>(tile_args(s, false), ad);
-    return cudaGetLastError();
+    return launch_in_chain(s.chained, step2d_u2_kernel<false, false, true>, grid, kUThreads, st, tile_args(s, false), ad);
 }
 
 bool step2_f16neq_enabled()

@@ -17,6 +17,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "lbrs_chain.cuh"
 #include "lbrs_kernels.cuh"
 #include "lbrs_launch.h"
 
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(32, kFMBlocks) fmarch_kernel(const FMarchArgs 
     float h1[2][4], h2[2][4];           // f_2, f_3 of the rows r - 1 and r - 2, as their receivers see them
 #pragma unroll
     for (int k = 0; k < 4; ++k) h1[0][k] = h1[1][k] = h2[0][k] = h2[1][k] = 0.f;
+    chain_begin();
     load(ja - 1);
 #pragma unroll 1
     for (int r = ja - 1; r <= jb; ++r) {
@@ -208,7 +210,8 @@ static int fmarch_rows(int nx, int ny)
 // on tiles by plain loads 57.8, march 52.0).
 bool fmarch_beats_tiles(int nx, int ny) { return fmarch_wave_rows(nx, ny) <= 10; }
 
-cudaError_t launch_fmarch_f32(const StepArgs<float>& s, const float ghost[4][GHOST_STRIDE], cudaStream_t st)
+cudaError_t launch_fmarch_f32(const StepArgs<float>& s, const float ghost[4][GHOST_STRIDE], bool chained,
+                              cudaStream_t st)
 {
     FMarchArgs a;
     a.src = s.src;
@@ -231,13 +234,11 @@ cudaError_t launch_fmarch_f32(const StepArgs<float>& s, const float ghost[4][GHO
     a.rows = fmarch_rows(s.nx, s.ny);
     const dim3 grid((unsigned)strips, (unsigned)((s.ny + a.rows - 1) / a.rows));
     if (s.Uout) {
-        if (sides) fmarch_kernel<true, true><<<grid, 32, 0, st>>>(a);
-        else fmarch_kernel<false, true><<<grid, 32, 0, st>>>(a);
-    } else {
-        if (sides) fmarch_kernel<true, false><<<grid, 32, 0, st>>>(a);
-        else fmarch_kernel<false, false><<<grid, 32, 0, st>>>(a);
+        if (sides) return launch_in_chain(chained, fmarch_kernel<true, true>, grid, 32, st, a);
+        return launch_in_chain(chained, fmarch_kernel<false, true>, grid, 32, st, a);
     }
-    return cudaGetLastError();
+    if (sides) return launch_in_chain(chained, fmarch_kernel<true, false>, grid, 32, st, a);
+    return launch_in_chain(chained, fmarch_kernel<false, false>, grid, 32, st, a);
 }
 
 }  // namespace lbrs

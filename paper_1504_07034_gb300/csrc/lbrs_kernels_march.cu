@@ -224,13 +224,12 @@ double march_rows_for(MarchArgs& a, int own, int steps)
 }
 
 template <int K, bool RECORD>
-cudaError_t launch_k(MarchArgs a, cudaStream_t s)
+cudaError_t launch_k(MarchArgs a, bool chained, cudaStream_t s)
 {
     march_rows_for(a, MarchShape<K>::own, K);
     const int64_t blocks = (int64_t)a.strips * a.chunks;
-    if (a.nx & 1) march2d_kernel<K, true, RECORD><<<(unsigned)blocks, 32, 0, s>>>(a);
-    else march2d_kernel<K, false, RECORD><<<(unsigned)blocks, 32, 0, s>>>(a);
-    return cudaGetLastError();
+    if (a.nx & 1) return launch_in_chain(chained, march2d_kernel<K, true, RECORD>, (unsigned)blocks, 32, s, a);
+    return launch_in_chain(chained, march2d_kernel<K, false, RECORD>, (unsigned)blocks, 32, s, a);
 }
 
 }  // namespace
@@ -299,8 +298,8 @@ cudaError_t launch_march_f32(const MarchStep& st, int steps, bool record, cudaSt
     for (int n = 0; n < 4; ++n) a.bc[n] = st.bc[n];
     a.c = st.c;
     a.gm1 = st.gm1;
-    if (record) return steps == 2 ? launch_k<2, true>(a, s) : launch_k<1, true>(a, s);
-    return steps == 2 ? launch_k<2, false>(a, s) : launch_k<1, false>(a, s);
+    if (record) return steps == 2 ? launch_k<2, true>(a, st.chained, s) : launch_k<1, true>(a, st.chained, s);
+    return steps == 2 ? launch_k<2, false>(a, st.chained, s) : launch_k<1, false>(a, st.chained, s);
 }
 
 cudaError_t launch_pull_moments_f32(const StepArgs<float>& a, float* U, cudaStream_t s)

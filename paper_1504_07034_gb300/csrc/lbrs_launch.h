@@ -160,6 +160,7 @@ struct MarchStep {
     int nx, ny;
     int bc[4];
     float c, gm1;
+    bool chained;              // the next of a captured chain (lbrs_chain.cuh)
 };
 bool march_enabled();
 // The moments-only form's tile kernels (launch_step2_f32u) are faster on this grid; never with
@@ -234,6 +235,7 @@ struct F16StepArgs {
     int bc[4];
     float om, om1, c, gm1;
     const uint8_t* walls;  // launch_step2_f32u only: the cells' wall codes, or NULL without internal walls
+    bool chained;          // two-step launches: the next of a captured chain (lbrs_chain.cuh)
 };
 cudaError_t launch_step_f16neq(const F16StepArgs& a, cudaStream_t s);
 // The same, two steps per launch (bit-identical); off when the environment sets LBRS_F16_FUSE=0.
@@ -260,7 +262,8 @@ cudaError_t launch_adapt_leave_f32(const float* U, float* f, int64_t N, float gm
 bool adapt_moments_enabled();
 // FP32 distribution form, omega != 1: two steps per launch, marching (lbrs_kernels_fmarch.cu); a.Uout: both
 // steps' moments.  No internal walls, no halfway walls.  LBRS_F32_FMARCH=0 turns it off.
-cudaError_t launch_fmarch_f32(const StepArgs<float>& a, const float ghost[4][GHOST_STRIDE], cudaStream_t s);
+cudaError_t launch_fmarch_f32(const StepArgs<float>& a, const float ghost[4][GHOST_STRIDE], bool chained,
+                              cudaStream_t s);
 bool fmarch_enabled();
 bool fmarch_beats_tiles(int nx, int ny);
 cudaError_t launch_set_state_f32u(const void* W, int w_dtype, int kind, void* fs, int64_t N, int64_t plane,

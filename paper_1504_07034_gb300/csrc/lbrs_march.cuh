@@ -19,6 +19,7 @@
 // collide_2d, where the compiler contracts the same products.
 #pragma once
 
+#include "lbrs_chain.cuh"
 #include "lbrs_kernels.cuh"
 
 namespace lbrs {
@@ -401,6 +402,7 @@ __device__ __forceinline__ void march_rows(const MarchArgs& a, const MarchPlace&
 template <int K, bool ODD, bool RECORD>
 __global__ void __launch_bounds__(32, 16) march2d_kernel(const __grid_constant__ MarchArgs a)
 {
+    chain_begin();
     const int strip = blockIdx.x % a.strips;
     const int chunk = blockIdx.x / a.strips;
     int ya = chunk * a.rows, yb = min(ya + a.rows, a.ny);

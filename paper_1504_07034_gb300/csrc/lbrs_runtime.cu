@@ -274,6 +274,10 @@ StepArgs<T> step_args(const lbrs_ctx* ctx, int from)
 }
 
 // Arguments of the reduced-state kernels (FP16 non-equilibrium and moments-only forms).
+// Is s being captured into a graph of the library's own?  Its launches then chain (lbrs_chain.cuh); a
+// caller's capture gets ordinary ones.
+bool own_capture(const lbrs_ctx* ctx, cudaStream_t s) { return ctx->cap_stream && s == ctx->cap_stream; }
+
 F16StepArgs f16_args(const lbrs_ctx* ctx, int from)
 {
     F16StepArgs a;
@@ -289,6 +293,7 @@ F16StepArgs f16_args(const lbrs_ctx* ctx, int from)
     a.c = (float)ctx->c;
     a.gm1 = (float)(ctx->cfg.gamma - 1.0);
     a.walls = nullptr;
+    a.chained = false;
     return a;
 }
 
@@ -420,14 +425,20 @@ MarchStep march_step(const lbrs_ctx* ctx, const char* src, char* dst)
     for (int s = 0; s < 4; ++s) m.bc[s] = kernel_bc(ctx, s);
     m.c = (float)ctx->c;
     m.gm1 = (float)(ctx->cfg.gamma - 1.0);
+    m.chained = false;
     return m;
 }
 
 // m = 1 or 2 steps on the moments from src into dst.
 cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int m, cudaStream_t s)
 {
-    if (!ctx->mtiles && !ctx->solid) return launch_march_f32(march_step(ctx, src, dst), m, false, s);
+    if (!ctx->mtiles && !ctx->solid) {
+        MarchStep ms = march_step(ctx, src, dst);
+        ms.chained = own_capture(ctx, s);
+        return launch_march_f32(ms, m, false, s);
+    }
     F16StepArgs a = f16_args(ctx, 0);
+    a.chained = own_capture(ctx, s);
     a.src = src;
     a.dst = dst;
     if (ctx->solid) {
@@ -464,10 +475,14 @@ cudaError_t launch_step3(const lbrs_ctx* ctx, int b, cudaStream_t s)
 // Two steps from buffer b into buffer b ^ 1.
 cudaError_t launch_step2(const lbrs_ctx* ctx, int b, cudaStream_t s)
 {
-    if (ctx->f32u) return launch_step2_f32u(f16_args(ctx, b), s);
-    if (ctx->f16) return launch_step2_f16neq(f16_args(ctx, b), s);
+    const bool chained = own_capture(ctx, s);     // a graph of the library's own
+    if (ctx->f32u || ctx->f16) {
+        F16StepArgs a = f16_args(ctx, b);
+        a.chained = chained;
+        return ctx->f32u ? launch_step2_f32u(a, s) : launch_step2_f16neq(a, s);
+    }
     if (fused2_scalar(ctx)) return launch_step2s_f32(step_args<float>(ctx, b), s);
-    if (fmarch(ctx)) return launch_fmarch_f32(step_args<float>(ctx, b), ctx->mghost, s);
+    if (fmarch(ctx)) return launch_fmarch_f32(step_args<float>(ctx, b), ctx->mghost, chained, s);
     return launch_step2_f32(step_args<float>(ctx, b), &ctx->tmap[b], wait_flag(ctx), s);
 }
 
@@ -710,7 +725,7 @@ cudaError_t launch_record_step2(lbrs_ctx* ctx, void* Uout)
 {
     StepArgs<float> a = step_args<float>(ctx, ctx->cur);
     a.Uout = (float*)Uout;
-    if (fmarch(ctx)) return launch_fmarch_f32(a, ctx->mghost, ctx->stream);
+    if (fmarch(ctx)) return launch_fmarch_f32(a, ctx->mghost, false, ctx->stream);
     return launch_step2_f32(a, &ctx->tmap[ctx->cur], wait_flag(ctx), ctx->stream);
 }
 
