@@ -181,14 +181,25 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
     store(3);
 }
 
-// Rows a warp stores.  Fewer rows mean more warps to hide latencies, and more rows recomputed
-// around each warp's own (2 K of them).  An iteration (K source rows) takes 0.33 us by itself and
-// 0.17 us of an SM sub-partition's issue slots (K = 2, measured on 1024^2 and 4096 x 1024), so with w
-// warps on the fullest sub-partition a launch takes about (rows + 2 K) max(0.33, 0.17 w) us; the rule
-// takes the minimum over the rows (1024^2: 16 rows 10.1 us, 8 rows 11.0, 30 rows 15.3; 4096 x 1024:
-// 30 rows 29.3, 12 rows 31.8).  The warps beside y sides that are not periodic take longer per row
-// (0.40 us by themselves, 0.60 beside a wall) and get as many rows as keep them from ending last.
-// Returns that time.
+// Time of an iteration (K source rows) with w warps per SM sub-partition, in us (periodic, K = 2: 768^2
+// 0.34 at one on the fullest, 900^2 0.44 at two, 2048 x 512 0.63 at three, 1200^2 0.81 at four, 1.02 at
+// five), full waves and a rest beyond.
+double march_iteration(double w)
+{
+    static const double t[5] = {0.34, 0.34, 0.44, 0.63, 0.80};
+    if (w <= 4.0) return t[(int)ceil(w)];
+    double sum = 0.0;
+    for (; w > 4.0; w -= 4.0) sum += t[4];
+    return sum + 0.12 + 0.2 * w;
+}
+
+// Rows a warp stores.  Fewer rows mean more warps to hide latencies, and more rows recomputed around
+// each warp's own (2 K of them): a launch takes about 1.5 us and (rows + 2 K) iterations, and the rule
+// takes the minimum over the rows (us per step, K = 2: 1024^2 with clamped sides 16 rows 5.4, 10 rows
+// 6.2, 30 rows 7.1; 2048^2 30 rows in one full wave 16.2, 16 rows 17.5, 20 rows 18.0, 40 rows 17.3).
+// The warps beside y sides that are not periodic take longer per row (0.40 us by themselves, 0.60 beside
+// a wall, 0.4 more with another warp) and get as many rows, an even number, as keep them from ending
+// last (1024^2, 16 rows, 8 of them 5.4, 9 5.6, 12 6.2).  Returns that time without the 1.5 us.
 double march_rows_for(MarchArgs& a, int own, int steps)
 {
     a.strips = (a.nx + own - 1) / own;
@@ -199,15 +210,15 @@ double march_rows_for(MarchArgs& a, int own, int steps)
         int end = 0;
         int64_t chunks = (a.ny + rows - 1) / rows;
         const int64_t per_sm = (a.strips * chunks + kSMs - 1) / kSMs;
-        const double sub = per_sm <= kWarpsPerSM ? (double)((per_sm + 3) / 4) : (double)per_sm / 4.0 + 0.5;
-        const double resident = fmin(sub, kWarpsPerSM / 4);
-        double t = (rows + 2 * steps) * fmax(0.33, 0.17 * sub);
+        const double w = (double)per_sm / 4.0, resident = fmin(w, kWarpsPerSM / 4);
+        double t = (rows + 2 * steps) * march_iteration(w);
         if (!per) {
-            const double iteration = lone + 0.17 * (resident - 1.0);     // beside a y side
-            end = (int)((rows + 2 * steps) * fmax(0.33, 0.17 * resident) / iteration) - steps;
-            end = end < 2 ? 2 : (end > rows ? rows : end);
+            const double iteration = lone + 0.36 * fmin(fmax(ceil(resident) - 1.0, 0.0), 1.67);   // beside a y side
+            end = (int)((rows + 2 * steps) * march_iteration(resident) / iteration) - steps;
+            end = end < 2 ? 2 : (end > rows ? rows : end & ~1);
             if (a.ny > 2 * end) {
                 chunks = 2 + (a.ny - 2 * end + rows - 1) / rows;
+                t = (rows + 2 * steps) * march_iteration((double)((a.strips * chunks + kSMs - 1) / kSMs) / 4.0);
             } else {
                 end = 0;
                 t = fmax(t, (rows + steps) * iteration);
@@ -247,8 +258,8 @@ bool march_enabled() { return march_mode() != 0; }
 
 // The tile kernel's two-step launch (step2d_u2_kernel, 32 x 16 tiles, four blocks per SM) starts
 // faster than a march and wins on small grids: about 2.7 us and 1.05 us per tile of an SM against the
-// march's 3 us and its own time, a quarter more of it beside sides that are not periodic (per launch,
-// in a graph: 128^2 3.7 against 4.4 us periodic and 5.4 with clamped sides, 384^2 4.5 against 5.6 and
+// march's 1.5 us and its iterations, 1 us and a quarter more of them beside sides that are not periodic
+// (per launch, in a graph: 128^2 3.7 against 4.4 us periodic and 5.4 with clamped sides, 384^2 4.5 against 5.6 and
 // 6.5, 512^2 6.7 against 5.6 and 6.6, 1531 x 200 6.9 against 6.4 and 10.0, 768^2 10.7 against 7.9 and
 // 8.8).
 bool march_prefers_tiles(int nx, int ny, const int bc[4])
@@ -258,7 +269,8 @@ bool march_prefers_tiles(int nx, int ny, const int bc[4])
     a.nx = nx;
     a.ny = ny;
     for (int s = 0; s < 4; ++s) a.bc[s] = bc[s];
-    const double march = 3.0 + march_rows_for(a, MarchShape<2>::own, 2) * (bc[2] == BC_PERIODIC ? 1.0 : 1.25);
+    const bool per = bc[2] == BC_PERIODIC;
+    const double march = (per ? 1.5 : 2.5) + march_rows_for(a, MarchShape<2>::own, 2) * (per ? 1.0 : 1.25);
     const double tiles = (double)((nx + 31) / 32) * (double)((ny + 15) / 16);
     return 2.7 + 1.05 * tiles / kSMs < march;
 }
