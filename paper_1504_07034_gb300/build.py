@@ -55,8 +55,7 @@ UNITS = {
 }
 HEADERS = [CSRC / "lbrs_kernels.cuh", CSRC / "lbrs_batch.cuh", CSRC / "lbrs_march.cuh", CSRC / "lbrs_tube.cuh",
            CSRC / "lbrs_scalar.cuh", CSRC / "lbrs_adapt.cuh", CSRC / "lbrs_chain.cuh",
-           CSRC / "lbrs_fp64.cuh", CSRC / "lbrs_launch.h",
-           INCLUDE / "lbrs.h"]
+           CSRC / "lbrs_fold.cuh", CSRC / "lbrs_fp64.cuh", CSRC / "lbrs_launch.h", INCLUDE / "lbrs.h"]
 
 
 def nvcc() -> str:

@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "lbrs_kernels.cuh"
+#include "lbrs_fold.cuh"
 #include "lbrs_fp64.cuh"
 #include "lbrs_batch.cuh"
 #include "lbrs_launch.h"
@@ -264,28 +265,10 @@ __global__ void __launch_bounds__(kThreads) diag_partial_kernel(const Ts* __rest
     }
 }
 
-__global__ void diag_final_kernel(const double* __restrict__ partials, int nblocks, double cell_volume,
-                                  double* __restrict__ out)
+__global__ void __launch_bounds__(kFoldThreads) diag_final_kernel(const double* __restrict__ partials, int nblocks,
+                                                                  double cell_volume, double* __restrict__ out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double tot[4] = {0.0, 0.0, 0.0, 0.0};
-    double mn_r = INFINITY, mn_p = INFINITY, mx_l = 0.0, nb = 0.0, ns = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
-        const double* p = partials + (int64_t)b * DIAG_W;
-        for (int k = 0; k < 4; ++k) tot[k] += p[k];
-        mn_r = fmin(mn_r, p[4]);
-        mn_p = fmin(mn_p, p[5]);
-        mx_l = fmax(mx_l, p[6]);
-        nb += p[7];
-        ns += p[8];
-    }
-    for (int k = 0; k < 4; ++k) out[k] = tot[k] * cell_volume;
-    out[4] = mn_r;
-    out[5] = mn_p;
-    out[6] = mx_l;
-    out[7] = nb;
-    out[8] = ns;
-    out[9] = 0.0;
+    fold_diag_records(partials, nblocks, cell_volume, out);
 }
 
 template <typename Ts, typename Tin>
@@ -329,12 +312,11 @@ __global__ void __launch_bounds__(kThreads) density_loss_kernel(int Q, int K, co
     }
 }
 
-__global__ void sum_final_kernel(const double* __restrict__ partials, int n, double scale, double* __restrict__ out)
+__global__ void __launch_bounds__(kFoldThreads) sum_final_kernel(const double* __restrict__ partials, int n, double scale,
+                                                                 double* __restrict__ out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-    for (int b = 0; b < n; ++b) s += partials[b];
-    out[0] = s * scale;
+    const double s = fold_sum(partials, n);
+    if (threadIdx.x == 0) out[0] = s * scale;
 }
 
 // Batched tubes: f = f^eq(U(W)) with the cell's own tube lambda, in FP64.
@@ -681,7 +663,7 @@ cudaError_t launch_density_loss(int Q, int K, int storage_f64, const void* fs, c
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    sum_final_kernel<<<1, 32, 0, s>>>(partials, g, cell_volume, out);
+    sum_final_kernel<<<1, kFoldThreads, 0, s>>>(partials, g, cell_volume, out);
     return cudaGetLastError();
 }
 
@@ -794,7 +776,7 @@ cudaError_t launch_diag(int lattice, int storage_f64, const void* fs, int64_t N,
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    diag_final_kernel<<<1, 32, 0, s>>>(partials, kDiagBlocks, cell_volume, out);
+    diag_final_kernel<<<1, kFoldThreads, 0, s>>>(partials, kDiagBlocks, cell_volume, out);
     return cudaGetLastError();
 }
 

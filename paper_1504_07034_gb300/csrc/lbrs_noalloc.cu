@@ -36,6 +36,7 @@
 #include <cuda_runtime.h>
 
 #include "lbrs.h"
+#include "lbrs_fold.cuh"
 #include "lbrs_kernels.cuh"
 
 namespace lbrs {
@@ -163,30 +164,10 @@ __global__ void __launch_bounds__(kThreads) noalloc_partial_kernel(const Ts* __r
     }
 }
 
-// Folds the nblocks records in block order into the result slot after the
-// last possible record.
-__global__ void noalloc_final_kernel(int nblocks, double cell_volume)
+// Folds the nblocks records into the result slot after the last possible record.
+__global__ void __launch_bounds__(kFoldThreads) noalloc_final_kernel(int nblocks, double cell_volume)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double tot[4] = {0.0, 0.0, 0.0, 0.0};
-    double mn_r = INFINITY, mn_p = INFINITY, mx_l = 0.0, nb = 0.0, ns = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
-        const double* p = g_diag_scratch + (int64_t)b * DIAG_W;
-        for (int k = 0; k < 4; ++k) tot[k] += p[k];
-        mn_r = fmin(mn_r, p[4]);
-        mn_p = fmin(mn_p, p[5]);
-        mx_l = fmax(mx_l, p[6]);
-        nb += p[7];
-        ns += p[8];
-    }
-    double* out = g_diag_scratch + (int64_t)kMaxBlocks * DIAG_W;
-    for (int k = 0; k < 4; ++k) out[k] = tot[k] * cell_volume;
-    out[4] = mn_r;
-    out[5] = mn_p;
-    out[6] = mx_l;
-    out[7] = nb;
-    out[8] = ns;
-    out[9] = 0.0;
+    fold_diag_records(g_diag_scratch, nblocks, cell_volume, g_diag_scratch + (int64_t)kMaxBlocks * DIAG_W);
 }
 
 // Device address of the scratch on the current device, looked up once per device.
@@ -257,7 +238,7 @@ extern "C" lbrs_status lbrs_diagnostics_noalloc(const lbrs_config* cfg, const vo
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        noalloc_final_kernel<<<1, 32, 0, stream>>>(nblocks, vol);
+        noalloc_final_kernel<<<1, kFoldThreads, 0, stream>>>(nblocks, vol);
         e = cudaGetLastError();
     }
     double h[DIAG_W];
