@@ -385,10 +385,15 @@ bool step3_tiles(const lbrs_ctx* ctx)
     return ctx->tmap3[0].valid && ctx->tmap3[1].valid;
 }
 
+// Rows up to which one row a block still fits a launch grid; taller ones keep the tile kernels, whose
+// blocks take at least 12.
+constexpr int64_t kMaxGridY = 65535;
+
 // FP32 distributions at omega != 1 two steps a launch by the marching kernel (lbrs_kernels_fmarch.cu)?
 // The switches that ask for one or two storing steps a launch turn it off.
 bool fmarch(const lbrs_ctx* ctx)
 {
+    if (ctx->ny_store > kMaxGridY) return false;
     if (!fmarch_enabled() || !fused2_f32(ctx) || !step3_f32_enabled() || ctx->solid || ctx->cfg.omega == 1.0) return false;
     if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
     return !step3_tiles(ctx) || fmarch_beats_tiles((int)ctx->cfg.nx, (int)ctx->ny_store);
@@ -402,6 +407,7 @@ bool fused3(const lbrs_ctx* ctx) { return step3_tiles(ctx) && !fmarch(ctx); }
 // tile kernel (a fluid cell never uses what a solid cell holds), but not recording steps.
 bool on_moments(const lbrs_ctx* ctx)
 {
+    if (ctx->ny_store > kMaxGridY) return false;
     if (ctx->f64 || ctx->f16 || ctx->lattice != LBRS_D2Q4 || ctx->cfg.omega != 1.0) return false;
     if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
     return march_enabled() && (ctx->f32u ? step2_f32u_enabled() : step2_f32_enabled() && step3_f32_enabled());
@@ -454,9 +460,12 @@ cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int 
 int64_t march_min(const lbrs_ctx* ctx) { return ctx->N < 400000 ? 8 : 6; }
 
 // Steps the next launch takes out of `left`: three where the three-step kernel applies (but
-// 2 + 2 rather than 3 + 1), else two where the two-step kernel does, else one.
+// 2 + 2 rather than 3 + 1), else two where the two-step kernel does, else one.  Beside the marching
+// kernel's two the tiles' three take the last three (1024^2 at omega = 1.5 in calls of three steps, the
+// caches flushed before each: 70 GLUPS, as two and one 59).
 int next_launch_steps(const lbrs_ctx* ctx, int64_t left)
 {
+    if (left == 3 && step3_tiles(ctx)) return 3;
     if (left >= 3 && left != 4 && fused3(ctx)) return 3;
     if (left >= 2 && fused2(ctx)) return 2;
     return 1;
@@ -787,10 +796,16 @@ lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
         ctx->cur ^= 1;
         ctx->launches += 1;
     }
-    for (; m + 2 <= n && fused2_f32(ctx) && !ctx->solid; m += 2) {
+    for (; m + 2 <= n && !(n - m == 3 && step3_tiles(ctx)) && fused2_f32(ctx) && !ctx->solid; m += 2) {
         LBRS_CUDA(ctx, launch_record_step2(ctx, U_hist + m * stride));
         ctx->cur ^= 1;
         ctx->launches += 1;
+    }
+    if (n - m == 3 && step3_tiles(ctx)) {
+        LBRS_CUDA(ctx, launch_record_step3(ctx, U_hist + m * stride));
+        ctx->cur ^= 1;
+        ctx->launches += 1;
+        m += 3;
     }
     for (; m < n; ++m) {
         LBRS_CUDA(ctx, launch_record_step(ctx, U_hist + m * stride));

@@ -23,7 +23,7 @@ D0, D1 = ("dirichlet", (0.9, 0.6, -0.2, 0.8)), ("dirichlet", (1.1, -0.3, 0.4, 1.
 T, P, WL = ("transmissive", None), ("periodic", None), ("wall", None)
 SETS = [[P, P, P, P], [T, T, T, T], [D0, T, WL, D1], [P, P, WL, WL], [T, D1, D0, WL], [D1, D0, P, P], [T, T, P, P],
         [D0, D1, T, D0]]
-SHAPES = [(1, 2), (2, 3), (29, 2), (30, 5), (31, 4), (61, 33), (130, 47), (700, 645)]
+SHAPES = [(1, 2), (2, 3), (29, 2), (30, 5), (31, 4), (61, 33), (130, 47), (700, 645), (3, 65540)]
 rng = np.random.default_rng(9)
 out = []
 for bc in SETS:

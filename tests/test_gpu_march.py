@@ -27,7 +27,7 @@ SETS = [[P, P, P, P], [T, T, T, T], [("dirichlet", D0), T, WL, ("dirichlet", D1)
         [T, ("dirichlet", D1), ("dirichlet", D0), WL], [("dirichlet", D1), ("dirichlet", D0), P, P],
         [("dirichlet", D0), ("dirichlet", D1), T, ("dirichlet", D0)]]
 SHAPES = [(1, 1), (2, 3), (59, 2), (60, 5), (61, 4), (62, 7), (63, 9), (64, 33), (65, 40), (119, 6), (120, 64),
-          (121, 17), (257, 70), (1021, 13), (1200, 131)]
+          (121, 17), (257, 70), (1021, 13), (1200, 131), (3, 65540)]
 rng = np.random.default_rng(7)
 out = []
 for bc in SETS:
