@@ -560,7 +560,8 @@ def oblique_measurement(Solver, stream, barrier, peak):
     import torch
     out = {"workload": "oblique shock reflection 4096x1024, 200 timed steps per form, CUDA-graph replay, "
                        "working set larger than L2 (no flush needed)"}
-    for precision, bpl in (("f32", BYTES_PER_LUP_F32_FUSED3), ("f16neq", BYTES_PER_LUP_F16NEQ),
+    # FP32 at omega = 1 steps on the moments, 32 B per cell and two steps
+    for precision, bpl in (("f32", BYTES_PER_LUP_F32U / 2), ("f16neq", BYTES_PER_LUP_F16NEQ),
                            ("f32u", BYTES_PER_LUP_F32U)):
         big = workloads.from_config("oblique_shock_4096x1024", steps=216)[1]   # six 36-step graphs
         s = Solver.from_workload(big, precision=precision, stream=stream)
@@ -577,9 +578,9 @@ def oblique_measurement(Solver, stream, barrier, peak):
         mlups = big.cells * big.steps / t / 1e6
         out[precision] = {"value": mlups, "unit": UNIT, "algorithmic_bytes_per_lup": bpl,
                           "achieved_gbs": bpl * mlups / 1e3, "frac": bpl * mlups / 1e3 / peak}
-        if precision == "f32u":                 # two steps per launch: U read and written once per two steps
-            out[precision]["kernel_bytes_per_lup"] = 16
-            out[precision]["kernel_frac"] = 16 * mlups / 1e3 / peak
+        if precision != "f32":                  # two steps per launch: the state read and written once per two steps
+            out[precision]["kernel_bytes_per_lup"] = bpl // 2
+            out[precision]["kernel_frac"] = bpl // 2 * mlups / 1e3 / peak
         s.close()
     for omega, steps in ((1.0, 20000), (1.5, 2000)):
         wl = workloads.from_config("oblique_shock_4096x1024", steps=steps, omega=omega)[1]
@@ -662,14 +663,13 @@ def obstacle_measurement(Solver, stream, barrier, peak):
     s.close()
     t = a.elapsed_time(b) / 1e3
     mlups = big.cells * big.steps / t / 1e6
-    bpl = BYTES_PER_LUP_F32_FUSED2 + 0.5
+    bpl = BYTES_PER_LUP_F32U / 2 + 0.5
     out["steady_6144x2048_f32"] = {"value": mlups, "unit": UNIT,
-                                   "kernel": "step2d_f32_fused2_tall_kernel<false, true>",
+                                   "kernel": "step2d_u2_kernel<false, true, false>",
                                    "algorithmic_bytes_per_lup": bpl, "achieved_gbs": bpl * mlups / 1e3,
                                    "frac": bpl * mlups / 1e3 / peak,
-                                   "note": "two steps per launch with the obstacle mask of each tile's pull "
-                                           "range in shared memory: 128 B of distributions and the 1 B mask "
-                                           "per cell and launch"}
+                                   "note": "two steps per launch on the moments: 32 B of moments and the 1 B wall "
+                                           "code per cell and launch"}
     return out
 
 
@@ -712,12 +712,12 @@ def burgers_measurement(Solver, stream, barrier, peak):
     mlups = big.cells * big.steps / t / 1e6
     bpl = 32
     out["steady_8192x8192_f32"] = {"value": mlups, "unit": UNIT,
-                                   "kernel": "step2ds_fused2_kernel (two steps per launch)",
+                                   "kernel": "step2ds_window_kernel (eight steps per launch)",
                                    "algorithmic_bytes_per_lup": bpl, "achieved_gbs": bpl * mlups / 1e3,
                                    "frac": bpl * mlups / 1e3 / peak,
-                                   "kernel_bytes_per_lup": bpl // 2, "kernel_frac": bpl // 2 * mlups / 1e3 / peak,
+                                   "kernel_bytes_per_lup": 1, "kernel_frac": mlups / 1e3 / peak,
                                    "note": "frac against one read and one write of the 4 populations per step "
-                                           "(32 B), kernel_frac against the kernel's own 16 B per update"}
+                                           "(32 B), kernel_frac against u read and written once per eight steps"}
     return out
 
 
@@ -795,7 +795,7 @@ def batch_measurement(stream, barrier):
                        "autotune_ns_per_update": ns},
             "kernel_launches": launches,
             "d1q3": batch_d1q3_measurement(stream, barrier),
-            "note": "temporal blocking in shared memory: up to `halo` steps per launch, so the effective "
+            "note": "temporal blocking in registers: up to `halo` steps per launch, so the effective "
                     "48 B/LUP bandwidth can exceed the HBM peak"}
 
 

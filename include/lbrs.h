@@ -484,8 +484,9 @@ lbrs_status lbrs_backward_checkpointed(lbrs_ctx* ctx, void* d_adj_ws, const void
  * f[q][k][off_b + x], off_b = sum of the lengths of the tubes before b;
  * field arrays are [3][sum N_b].  The step per cell is the D1Q2 (or D1Q3,
  * cfg.lattice) step of Section II.C, identical in arithmetic to the single-tube path; the
- * kernels advance a tile of a tube by up to `halo` steps in shared memory per
- * launch (temporal blocking, see lbrs_batch_tuning). */
+ * kernels advance a tile of a tube by up to `halo` steps per launch, in
+ * registers (FP32, halo <= 64) or shared memory (temporal blocking, see
+ * lbrs_batch_tuning). */
 typedef struct lbrs_batch lbrs_batch;
 
 typedef struct {
@@ -503,7 +504,9 @@ typedef struct {
 /* Launch shape of the batched kernel: `block` threads (128, 256 or 512), each
  * owning `cells_per_thread` window cells; a window is block*cells_per_thread
  * cells, of which `halo` on each side are recomputed context and the rest
- * (the tile, >= 32 cells) is advanced by up to `halo` steps per launch. */
+ * (the tile, >= 32 cells) is advanced by up to `halo` steps per launch.  FP32
+ * tubes with halo <= 64 step in registers on windows of the kernel's own; of
+ * the tuning they take the halo (default 32). */
 typedef struct {
     int32_t block, cells_per_thread, halo, reserved;
 } lbrs_batch_tuning;
