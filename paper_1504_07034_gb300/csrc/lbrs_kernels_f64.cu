@@ -88,6 +88,21 @@ __device__ __forceinline__ void prim_to_cons(const double* w, double gamma, doub
     else prim_to_cons1d(w, gamma, U);
 }
 
+// The same with the division's reciprocal at hand: the same bits.
+template <int LAT>
+__device__ __forceinline__ void prim_to_cons(const double* w, const Fp64Divisor& gm1, double* U)
+{
+    U[0] = w[0];
+    if constexpr (LAT == LAT_D2Q4) {
+        U[1] = w[0] * w[1];
+        U[2] = w[0] * w[2];
+        U[3] = gm1.divide(w[3]) + 0.5 * w[0] * (w[1] * w[1] + w[2] * w[2]);
+    } else if constexpr (LAT != LAT_D2Q4S) {
+        U[1] = w[0] * w[1];
+        U[2] = gm1.divide(w[2]) + 0.5 * w[0] * (w[1] * w[1]);
+    }
+}
+
 template <typename Ts, int LAT>
 __global__ void ghost_kernel(GhostSpec g, double gamma, double c, Ts* ghost)
 {
@@ -117,12 +132,13 @@ __global__ void __launch_bounds__(kThreads) set_state_kernel(const Tin* __restri
                                                              double c)
 {
     constexpr int Q = Dims<LAT>::Q, K = Dims<LAT>::K;
+    const Fp64Divisor gm1(gamma - 1.0);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         double w[4], U[4], e[16];
 #pragma unroll
         for (int k = 0; k < K; ++k) w[k] = (double)W[k * N + i];
         if (kind == KIND_PRIMITIVE) {
-            prim_to_cons<LAT>(w, gamma, U);
+            prim_to_cons<LAT>(w, gm1, U);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k) U[k] = w[k];
@@ -326,6 +342,7 @@ __global__ void __launch_bounds__(kThreads) batch_set_state_kernel(const Tin* __
                                                                    const int64_t* __restrict__ tube_off, int64_t nb,
                                                                    const double* __restrict__ tube_lam, int q)
 {
+    const Fp64Divisor gm1(gamma - 1.0);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = nb - 1;             // last tube with off <= i
         while (lo < hi) {
@@ -337,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) batch_set_state_kernel(const Tin* __
 #pragma unroll
         for (int k = 0; k < 3; ++k) w[k] = (double)W[k * N + i];
         if (kind == KIND_PRIMITIVE) {
-            prim_to_cons1d(w, gamma, U);
+            prim_to_cons<LAT_D1Q2>(w, gm1, U);
         } else {
 #pragma unroll
             for (int k = 0; k < 3; ++k) U[k] = w[k];
