@@ -301,8 +301,10 @@ __device__ __forceinline__ void rebuild(const F16Args& a, float c, const float U
 // walls, by the cells' codes; solid cells are stepped like others and mean nothing (no fluid cell reads
 // them).  ADAPT: adaptive lambda (lbrs_adapt.cuh; no Dirichlet sides), the bounds of both new states.  Every
 // block takes the clock forward while its loads are under way: 4 of a launch's 19 us at 768 x 768 (the
-// bounds 2 us), against a launch of its own or a last block's turn at about as much.
-template <bool F16, bool WALLS, bool ADAPT>
+// bounds 2 us), against a launch of its own or a last block's turn at about as much.  EARLY: a thread's
+// loads of phase A go out together, for grids of at most one tile per SM, where nothing else hides them
+// (us per step: 128^2 1.78 and early 1.57, 200^2 1.84 and 1.60; 500^2 3.23 and 3.42).
+template <bool F16, bool WALLS, bool ADAPT, bool EARLY = ADAPT>
 __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const F16Args a, const AdaptPair ad)
 {
     __shared__ float4 s_f[4 * kAN];      // [q][slot], slot = wy * kAX + wx
@@ -325,22 +327,29 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     const float g32 = (float)ad.gamma;
     const unsigned slot8 = (blockIdx.x + blockIdx.y * gridDim.x) % kBoundSlots;
     bool skip2 = false;                                    // the second step lies beyond the run's end
-    if constexpr (ADAPT) {
-        // phase A, its loads under way while the first warp takes the clock forward
-        if (threadIdx.x < 2) s_max[threadIdx.x] = 0u;
-        __shared__ float s_c[2];
-        __shared__ int s_skip[2];
+    if constexpr (EARLY) {
+        // phase A, a thread's loads all under way before their equilibria (ADAPT: while the first warp takes
+        // the clock forward)
+        if (ADAPT && threadIdx.x < 2) s_max[threadIdx.x] = 0u;
         constexpr int kAPer = (kAN + kUThreads - 1) / kUThreads;
         float Ua[kAPer][4];
         bool any[kAPer];
+        int side[kAPer];                                   // the Dirichlet side whose ghost the slot holds, or -1
 #pragma unroll
         for (int r = 0; r < kAPer; ++r) {
             const int w = threadIdx.x + r * kUThreads;
             int i = i0 + w % kAX, j = j0 + w / kAX;
             any[r] = w < kAN;
+            side[r] = -1;
             if (!inside) {
+                // two cells beyond a non-periodic side: only inner slots beyond that side would pull
+                // from here, and those are not gathered from their own position
                 const int bx = beyond(i, a.nx), by = beyond(j, a.ny);
                 if ((bx > 1 && !per_x) || (by > 1 && !per_y) || bx > 2 || by > 2) any[r] = false;
+                if constexpr (!ADAPT) {
+                    if (by && (j < 0 ? a.bc[2] : a.bc[3]) == BC_DIRICHLET) side[r] = j < 0 ? 2 : 3;
+                    if (bx && (i < 0 ? a.bc[0] : a.bc[1]) == BC_DIRICHLET) side[r] = i < 0 ? 0 : 1;
+                }
                 if (bx) i = per_x ? wrap_mod(i, a.nx) : (i < 0 ? 0 : a.nx - 1);
                 if (by) j = per_y ? wrap_mod(j, a.ny) : (j < 0 ? 0 : a.ny - 1);
             }
@@ -348,34 +357,45 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
 #pragma unroll
             for (int k = 0; k < 4; ++k) Ua[r][k] = any[r] ? a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 47)] : 1.f;
         }
-        if (threadIdx.x < 32) {
-            AdaptRun r1, r2;
-            adapt_clocks(*ad.in, ad.bounds_in, ad.pending, ad.dx, ad.safety, ad.t_final, r1, r2);
-            if (threadIdx.x == 0) {
-                s_c[0] = (float)r1.c;
-                s_skip[0] = r1.done;
-                s_c[1] = (float)r2.c;
-                s_skip[1] = r2.done;
-                if (blockIdx.x == 0 && blockIdx.y == 0) *ad.out = r2;
+        if constexpr (ADAPT) {
+            __shared__ float s_c[2];
+            __shared__ int s_skip[2];
+            if (threadIdx.x < 32) {
+                AdaptRun r1, r2;
+                adapt_clocks(*ad.in, ad.bounds_in, ad.pending, ad.dx, ad.safety, ad.t_final, r1, r2);
+                if (threadIdx.x == 0) {
+                    s_c[0] = (float)r1.c;
+                    s_skip[0] = r1.done;
+                    s_c[1] = (float)r2.c;
+                    s_skip[1] = r2.done;
+                    if (blockIdx.x == 0 && blockIdx.y == 0) *ad.out = r2;
+                }
+                if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2 * kBoundSlots) ad.bounds_clear[threadIdx.x] = 0ull;
             }
-            if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2 * kBoundSlots) ad.bounds_clear[threadIdx.x] = 0ull;
-        }
-        __syncthreads();
-        c0 = s_c[0];
-        c1 = s_c[1];
-        skip2 = s_skip[1];
-        if (s_skip[0]) {                                   // both: the state stays
-            const int i = ti0 + (int)threadIdx.x % kUX, j = tj0 + (int)threadIdx.x / kUX;
-            if (i >= a.nx || j >= a.ny) return;
-            const int64_t c = (int64_t)j * a.nx + i;
+            __syncthreads();
+            c0 = s_c[0];
+            c1 = s_c[1];
+            skip2 = s_skip[1];
+            if (s_skip[0]) {                                   // both: the state stays
+                const int i = ti0 + (int)threadIdx.x % kUX, j = tj0 + (int)threadIdx.x / kUX;
+                if (i >= a.nx || j >= a.ny) return;
+                const int64_t c = (int64_t)j * a.nx + i;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 59)];
-            return;
+                for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 59)];
+                return;
+            }
         }
 #pragma unroll
         for (int r = 0; r < kAPer; ++r) {
             const int w = threadIdx.x + r * kUThreads;
             if (!any[r]) continue;
+            if (!ADAPT && side[r] >= 0) {
+                const float* g = a.ghost + side[r] * GHOST_STRIDE;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    s_f[LBRS_IX(q * kAN + w, 4 * kAN, 42)] = make_float4(g[q * 4], g[q * 4 + 1], g[q * 4 + 2], g[q * 4 + 3]);
+                continue;
+            }
             float e[4][4];
             equilibria2d<float>(Ua[r], a.gm1, c0, e);
 #pragma unroll
@@ -693,6 +713,8 @@ cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
     if (s.walls)
         return launch_in_chain(s.chained, step2d_u2_kernel<false, true, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
+    if ((int64_t)grid.x * grid.y <= 152)
+        return launch_in_chain(s.chained, step2d_u2_kernel<false, false, false, true>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
     return launch_in_chain(s.chained, step2d_u2_kernel<false, false, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
 }
 
