@@ -241,4 +241,6 @@ cudaError_t launch_fmarch_f32(const StepArgs<float>& s, const float ghost[4][GHO
     return launch_in_chain(chained, fmarch_kernel<false, false>, grid, 32, st, a);
 }
 
+LBRS_DEBUG_WORD(debug_word_fmarch)
+
 }  // namespace lbrs

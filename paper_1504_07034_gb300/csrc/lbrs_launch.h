@@ -37,6 +37,7 @@ unsigned long long debug_word_f32(int clear);
 unsigned long long debug_word_f64(int clear);
 unsigned long long debug_word_f16(int clear);
 unsigned long long debug_word_march(int clear);
+unsigned long long debug_word_fmarch(int clear);
 unsigned long long debug_word_tube(int clear);
 unsigned long long debug_word_scalar(int clear);
 

@@ -895,7 +895,7 @@ lbrs_status lbrs_debug_check(uint64_t* first)
     if (!first) return fail(nullptr, LBRS_EINVAL, "first is NULL");
     unsigned long long w = 0ull;
     for (unsigned long long v : {debug_word_f32(1), debug_word_f64(1), debug_word_f16(1), debug_word_march(1),
-                                 debug_word_tube(1), debug_word_scalar(1)})
+                                 debug_word_fmarch(1), debug_word_tube(1), debug_word_scalar(1)})
         if (!w) w = v;
     *first = (uint64_t)w;
     if (w)
