@@ -140,4 +140,20 @@ __device__ __forceinline__ void equilibria1d3<double>(const double U[3], double 
     }
 }
 
+// bound2d's local bound by one reciprocal of rho for its three quotients, the same bits (adaptive 768^2
+// step 157 us with the three divisions, 141 so).
+template <>
+__device__ __forceinline__ double bound_local<double>(const double U[4], double gamma)
+{
+    if (!fp64_mid_range(U[0]) || !fp64_quotient_ok(U[1]) || !fp64_quotient_ok(U[2])) return bound2d<double>(U, gamma);
+    const double gm1 = gamma - 1.0;
+    const double y = fp64_reciprocal(U[0]);
+    const double u = fp64_quotient(U[1], U[0], y), v = fp64_quotient(U[2], U[0], y);
+    const double p = gm1 * __fma_rn(-0.5, U[1] * u + U[2] * v, U[3]);
+    const double gp = gamma * p;
+    if (!(U[0] > 0.0) || !(p > 0.0) || !isfinite(p)) return -1.0;
+    const double a = sqrt(fp64_mid_range(gp) ? fp64_quotient(gp, U[0], y) : gp / U[0]);
+    return fabs(u) + fabs(v) + sqrt(2.0) * a;
+}
+
 }  // namespace lbrs
