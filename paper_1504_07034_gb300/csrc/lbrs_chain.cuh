@@ -5,8 +5,14 @@
 // (1024 x 1024 on the moments 5.8 us per step unchained, 5.7 chained, 7.2 when asked for at the top).
 // 0.1 to 0.3 us of each launch (us per step, unchained and chained: internal walls at 960 x 320 3.97 and
 // 3.84, moments of 128^2 1.89 and 1.78, omega != 1 at 64^2 1.41 and 1.22, at 1000^2 11.5 and 11.35).
+//
+// A chained kernel is resident while the one before it still writes, so what that one writes is not
+// read-only for its lifetime: neither __ldg nor a plain load that the compiler may take for one (a const
+// __restrict__ pointer) may read it, because such loads go through the non-coherent path and may move
+// above the wait.  chain_load reads it.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 namespace lbrs {
@@ -16,6 +22,27 @@ namespace lbrs {
 __device__ __forceinline__ void chain_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Loads of what the launch before wrote: coherent, and behind chain_begin (volatile statements keep their
+// order).
+__device__ __forceinline__ float chain_load(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned long long chain_load(const unsigned long long* p)
+{
+    unsigned long long v;
+    asm volatile("ld.global.b64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half chain_load(const __half* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
 }
 
 // Launch; chained: as the next of a chain whose every kernel begins with chain_begin.

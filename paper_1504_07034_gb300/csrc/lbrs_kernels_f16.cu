@@ -39,13 +39,13 @@ namespace lbrs {
 namespace {
 
 struct F16Args {
-    const float* __restrict__ Uin;     // [4][N]
-    const __half* __restrict__ gin;    // [3][4][N]
-    float* __restrict__ Uout;
-    __half* __restrict__ gout;
+    const float* Uin;                  // [4][N]
+    const __half* gin;                 // [3][4][N]
+    float* Uout;
+    __half* gout;
     const float* __restrict__ ghost;   // [4][GHOST_STRIDE] full f of the Dirichlet states
-    const float* __restrict__ scale;   // [4] s_k, tail of the input buffer
-    float* __restrict__ scale_out;     // tail of the output buffer
+    const float* scale;                // [4] s_k, tail of the input buffer
+    float* scale_out;                  // tail of the output buffer
     int64_t N;
     int nx, ny;
     int bc[4];
@@ -313,10 +313,10 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     if constexpr (F16) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            sc[k] = a.scale[k];
+            sc[k] = chain_load(a.scale + k);
             inv[k] = 1.f / sc[k];          // exact: the scales are powers of two
         }
-        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) a.scale_out[threadIdx.x] = a.scale[threadIdx.x];
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) a.scale_out[threadIdx.x] = chain_load(a.scale + threadIdx.x);
     }
     const int ti0 = blockIdx.x * kUX, tj0 = blockIdx.y * kUY;
     const int i0 = ti0 - 2, j0 = tj0 - 2;                  // global cell of window slot (0, 0)
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
             }
             const int64_t c = (int64_t)j * a.nx + i;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) Ua[r][k] = any[r] ? a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 47)] : 1.f;
+            for (int k = 0; k < 4; ++k) Ua[r][k] = any[r] ? chain_load(a.Uin + LBRS_IX(k * a.N + c, 4 * a.N, 47)) : 1.f;
         }
         if constexpr (ADAPT) {
             __shared__ float s_c[2];
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
                 if (i >= a.nx || j >= a.ny) return;
                 const int64_t c = (int64_t)j * a.nx + i;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 59)];
+                for (int k = 0; k < 4; ++k) a.Uout[LBRS_IX(k * a.N + c, 4 * a.N, 59)] = chain_load(a.Uin + LBRS_IX(k * a.N + c, 4 * a.N, 59));
                 return;
             }
         }
@@ -436,15 +436,15 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
         const int64_t c = (int64_t)j * a.nx + i;
         float U[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) U[k] = a.Uin[LBRS_IX(k * a.N + c, 4 * a.N, 43)];
+        for (int k = 0; k < 4; ++k) U[k] = chain_load(a.Uin + LBRS_IX(k * a.N + c, 4 * a.N, 43));
         __half2 g[3][2];
         if constexpr (F16) {
 #pragma unroll
             for (int q = 0; q < 3; ++q)
 #pragma unroll
                 for (int k = 0; k < 4; k += 2)
-                    g[q][k / 2] = __halves2half2(a.gin[LBRS_IX((q * 4 + k) * a.N + c, 12 * a.N, 43)],
-                                                 a.gin[LBRS_IX((q * 4 + k + 1) * a.N + c, 12 * a.N, 43)]);
+                    g[q][k / 2] = __halves2half2(chain_load(a.gin + LBRS_IX((q * 4 + k) * a.N + c, 12 * a.N, 43)),
+                                                 chain_load(a.gin + LBRS_IX((q * 4 + k + 1) * a.N + c, 12 * a.N, 43)));
         }
         float e[4][4];
         rebuild<F16>(a, c0, U, g, sc, e);

@@ -28,9 +28,9 @@ constexpr int kFMOwn = 30;            // columns a warp stores
 constexpr int kFMBlocks = 24;         // warps of an SM (80 registers a lane)
 
 struct FMarchArgs {
-    const float* __restrict__ src;
-    float* __restrict__ dst;
-    float* __restrict__ Uout;         // recording: the moments of both steps, [2][4][N]
+    const float* src;
+    float* dst;
+    float* Uout;                      // recording: the moments of both steps, [2][4][N]
     float ghost[4][GHOST_STRIDE];     // f^eq of each Dirichlet side's state
     int64_t N;
     int nx, ny, rows;
@@ -119,22 +119,22 @@ __global__ void __launch_bounds__(32, kFMBlocks) fmarch_kernel(const FMarchArgs 
 
     // Beyond a clamped side a row is the side's own, computed once more.
     auto row_of = [&](int j) { return yper ? (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j)) : min(max(j, 0), a.ny - 1); };
+    chain_begin();
     float f[4][4];
     auto load = [&](int r) {
         const int j = row_of(r);
         const int64_t up = (int64_t)row_of(j + 1) * a.nx, down = (int64_t)row_of(j - 1) * a.nx;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            f[0][k] = __ldg(a.src + LBRS_IX((0 + k) * a.N + up + xp, 16 * a.N, 61));
-            f[1][k] = __ldg(a.src + LBRS_IX((4 + k) * a.N + up + xm, 16 * a.N, 61));
-            f[2][k] = __ldg(a.src + LBRS_IX((8 + k) * a.N + down + xm, 16 * a.N, 61));
-            f[3][k] = __ldg(a.src + LBRS_IX((12 + k) * a.N + down + xp, 16 * a.N, 61));
+            f[0][k] = chain_load(a.src + LBRS_IX((0 + k) * a.N + up + xp, 16 * a.N, 61));
+            f[1][k] = chain_load(a.src + LBRS_IX((4 + k) * a.N + up + xm, 16 * a.N, 61));
+            f[2][k] = chain_load(a.src + LBRS_IX((8 + k) * a.N + down + xm, 16 * a.N, 61));
+            f[3][k] = chain_load(a.src + LBRS_IX((12 + k) * a.N + down + xp, 16 * a.N, 61));
         }
     };
     float h1[2][4], h2[2][4];           // f_2, f_3 of the rows r - 1 and r - 2, as their receivers see them
 #pragma unroll
     for (int k = 0; k < 4; ++k) h1[0][k] = h1[1][k] = h2[0][k] = h2[1][k] = 0.f;
-    chain_begin();
     load(ja - 1);
 #pragma unroll 1
     for (int r = ja - 1; r <= jb; ++r) {

@@ -85,8 +85,8 @@ struct MarchShape {
 };
 
 struct MarchArgs {
-    const float* __restrict__ src;    // U [4][N]
-    float* __restrict__ dst;          // U [4][N], not src; RECORD: the moments of each step, [K][4][N]
+    const float* src;                 // U [4][N]
+    float* dst;                       // U [4][N], not src; RECORD: the moments of each step, [K][4][N]
     float ghost[4][GHOST_STRIDE];     // f^eq of each Dirichlet side's state, [q * 4 + k]
     int64_t N;                        // plane stride
     int nx, ny;
@@ -253,8 +253,8 @@ __device__ __forceinline__ P2 march_bottom(P2 S, const MarchArgs& a, const March
 template <bool ODD>
 __device__ __forceinline__ P2 march_load2(const float* p, int64_t n, int64_t row, const int x[2])
 {
-    if constexpr (ODD) return pk(__ldg(p + LBRS_IX(row + x[0], n, 51)), __ldg(p + LBRS_IX(row + x[1], n, 51)));
-    else return __ldg(reinterpret_cast<const P2*>(p + LBRS_IX(row + x[0], n - 1, 51)));
+    if constexpr (ODD) return pk(chain_load(p + LBRS_IX(row + x[0], n, 51)), chain_load(p + LBRS_IX(row + x[1], n, 51)));
+    else return chain_load(reinterpret_cast<const P2*>(p + LBRS_IX(row + x[0], n - 1, 51)));
 }
 
 template <bool ODD>
