@@ -1,6 +1,7 @@
 // FP32 D2Q4 steps at omega = 1 on the moments (lbrs_march.cuh): the launchers and the kernels
 // that lead from stored distributions into the moments and back.
 #include <math.h>
+#include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -239,7 +240,10 @@ cudaError_t launch_k(MarchArgs a, bool chained, cudaStream_t s)
 {
     march_rows_for(a, MarchShape<K>::own, K);
     const int64_t blocks = (int64_t)a.strips * a.chunks;
-    if (a.nx & 1) return launch_in_chain(chained, march2d_kernel<K, true, RECORD>, (unsigned)blocks, 32, s, a);
+    // pairs of columns move as 8-byte words where every row starts on one: nx even, and (moments recorded into
+    // a caller's buffer) the buffers themselves on 8 bytes
+    const bool words = (a.nx & 1) || (((uintptr_t)a.src | (uintptr_t)a.dst) & 7);
+    if (words) return launch_in_chain(chained, march2d_kernel<K, true, RECORD>, (unsigned)blocks, 32, s, a);
     return launch_in_chain(chained, march2d_kernel<K, false, RECORD>, (unsigned)blocks, 32, s, a);
 }
 

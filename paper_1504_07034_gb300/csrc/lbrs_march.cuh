@@ -175,8 +175,8 @@ struct MarchIn {
 
 // EDGE: the warp's window reaches an x side, and the end column takes its own value (clamped, EDGE = 1)
 // or, beside a Dirichlet side, the side's ghost (EDGE = 2), by selects: a branch or a load here would
-// cut the row's code into pieces that wait for one shuffle each.  ODD: nx is odd, and column nx - 1
-// may be the first of a lane.
+// cut the row's code into pieces that wait for one shuffle each.  ODD: column nx - 1 may be the first of
+// a lane (nx odd), and memory is accessed by single words.
 template <int EDGE, bool ODD, int K>
 __device__ __forceinline__ void march_shift(const P2 e[4], const MarchArgs& a, const MarchPlace& w, MarchIn& n)
 {
