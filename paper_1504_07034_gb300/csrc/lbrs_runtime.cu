@@ -1055,15 +1055,23 @@ lbrs_status lbrs_set_state(lbrs_ctx* ctx, const void* W, int on_device, int dtyp
 
 static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n);
 
+// Steps with the configured lambda do not continue an adaptive run's distributions.
+static lbrs_status fixed_lambda(lbrs_ctx* ctx)
+{
+    if (ctx->adapt_used)
+        return fail(ctx, LBRS_ESTATE, "the distributions carry an adaptive lambda: continue with "
+                                      "lbrs_step_adaptive or set a state");
+    return LBRS_OK;
+}
+
 lbrs_status lbrs_step(lbrs_ctx* ctx, int64_t n)
 {
     NvtxRange range("lbrs_step");
     if (!ctx) return fail(nullptr, LBRS_EINVAL, "ctx is NULL");
     if (n < 0) return fail(ctx, LBRS_EINVAL, "negative step count");
     if (!ctx->has_state) return fail(ctx, LBRS_ESTATE, "no state set");
-    if (ctx->adapt_used)
-        return fail(ctx, LBRS_ESTATE, "the distributions carry an adaptive lambda: continue with "
-                                      "lbrs_step_adaptive or set a state");
+    lbrs_status as = fixed_lambda(ctx);
+    if (as != LBRS_OK) return as;
     for (int h = 0; h < 2; ++h)
         if (ctx->halo[h] && n > ctx->halo_left[h])
             return fail(ctx, LBRS_ESTATE, "%lld steps requested, but the ghost rows of the %s cut cover %lld more "
@@ -1883,6 +1891,8 @@ lbrs_status lbrs_forward_checkpointed(lbrs_ctx* ctx, int64_t n_steps, int64_t se
     if (bytes < A.total) return fail(ctx, LBRS_ENOMEM, "adjoint workspace has %zu bytes, needs %zu", bytes, A.total);
     char* ws = (char*)d_adj_ws;
     ctx->adj_ws = nullptr;
+    st = fixed_lambda(ctx);
+    if (st != LBRS_OK) return st;
     ctx->adj_step0 = ctx->step;
     // at omega = 1 the run stays on the moments from its first step on: a checkpoint after the first
     // holds them (16 instead of 64 B per cell), written by the launch that ends its segment
