@@ -760,20 +760,22 @@ lbrs_status record_march(lbrs_ctx* ctx, const char* src, int64_t n, char* U_hist
     return LBRS_OK;
 }
 
-// The moments of the first step from the stored distributions f, into U.
+// The moments of the first step from the stored distributions f, into U (march: without internal walls,
+// also where a mask was set after the forward run that f belongs to).
 cudaError_t launch_pull_into(lbrs_ctx* ctx, const char* f, char* U)
 {
     StepArgs<float> a = step_args<float>(ctx, ctx->cur);
     a.src = (const float*)f;
+    a.solid = nullptr;
     ctx->launches += 1;
     return launch_pull_moments_f32(a, (float*)U, ctx->stream);
 }
 
-// The current buffer's distributions from the moments U at omega = 1.
-cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U)
+// The current buffer's distributions from the moments U at omega = 1, but those of the cells of `solid`.
+cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U, const uint8_t* solid)
 {
     ctx->launches += 1;
-    return launch_equilibria_f32((const float*)U, (float*)ctx->f[ctx->cur], ctx->solid, ctx->N, (float)ctx->c,
+    return launch_equilibria_f32((const float*)U, (float*)ctx->f[ctx->cur], solid, ctx->N, (float)ctx->c,
                                  (float)(ctx->cfg.gamma - 1.0), ctx->stream);
 }
 
@@ -787,7 +789,7 @@ lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
         LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], U_hist));
         lbrs_status st = record_march(ctx, U_hist, n - 1, U_hist + stride);
         if (st != LBRS_OK) return st;
-        LBRS_CUDA(ctx, launch_equilibria_from(ctx, U_hist + (n - 1) * stride));
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, U_hist + (n - 1) * stride, nullptr));
         return LBRS_OK;
     }
     int64_t m = 0;
@@ -1141,7 +1143,7 @@ static lbrs_status step_march(lbrs_ctx* ctx, int64_t n, bool graphs)
     if (ctx->f32u) {
         ctx->cur ^= rest & 1;
     } else {
-        LBRS_CUDA(ctx, launch_equilibria_from(ctx, v[rest & 1]));
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, v[rest & 1], ctx->solid));
     }
     ctx->step += n;
     ctx->launches += launches;
@@ -1920,7 +1922,7 @@ lbrs_status lbrs_forward_checkpointed(lbrs_ctx* ctx, int64_t n_steps, int64_t se
                 done += m;
             }
         }
-        LBRS_CUDA(ctx, launch_equilibria_from(ctx, at));
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, at, nullptr));
         ctx->step += n_steps;
     } else {
         for (int64_t s = 0; s < A.nseg; ++s) {
@@ -2016,7 +2018,7 @@ lbrs_status lbrs_backward_checkpointed(lbrs_ctx* ctx, void* d_adj_ws, const void
     // restore the final forward state
     const char* final_state = ws + A.ckpt0 + A.nseg * A.ckpt_stride;
     if (ctx->adj_moments)
-        LBRS_CUDA(ctx, launch_equilibria_from(ctx, final_state));
+        LBRS_CUDA(ctx, launch_equilibria_from(ctx, final_state, nullptr));
     else
         LBRS_CUDA(ctx, cudaMemcpyAsync(ctx->f[ctx->cur], final_state, ctx->L.f_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
     ctx->step = ctx->adj_step0 + ctx->adj_n;

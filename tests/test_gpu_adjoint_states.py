@@ -28,3 +28,24 @@ def test_adaptive_distributions_are_refused(precision, omega):
         s.forward_checkpointed(9, 3)
     assert e.value.status == abi.LBRS_ESTATE
     s.close()
+
+
+def test_mask_set_between_forward_and_backward():
+    """The backward pass is the forward run's: a mask set after it changes neither the gradient nor the
+    state that the backward pass puts back, in the mask's cells as in the others."""
+    res = []
+    for masked in (False, True):
+        s = _solver()
+        s.forward_checkpointed(11, 4)
+        end = s.raw_state().cpu().numpy()
+        _, g = s.vjp_loss(torch.ones(NY, NX, dtype=torch.float64, device="cuda"))
+        s.step(5)
+        if masked:
+            solid = torch.zeros(NY, NX, dtype=torch.uint8)
+            solid[10:20, 12:30] = 1
+            s.set_obstacles(solid)
+        grad = s.backward_checkpointed(g).cpu().numpy()
+        assert np.array_equal(s.raw_state().cpu().numpy(), end)
+        res.append(grad)
+        s.close()
+    assert np.array_equal(res[0], res[1])
