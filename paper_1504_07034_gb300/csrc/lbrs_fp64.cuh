@@ -3,12 +3,13 @@
 //
 // The FP64 path is bound by the chip's few FP64 units (about two operations per clock and SM), so an
 // operation saved is time saved:
-//  * both velocities share the reciprocal of rho: an approximate reciprocal refined by Newton-Raphson
-//    steps, the quotient m y corrected by its remainder, q' = q + (m - rho q) y.  With y the correctly
-//    rounded reciprocal, q' is the correctly rounded quotient (Markstein, "Computation of elementary
-//    functions on the IBM RISC System/6000 processor", 1990), that is the IEEE division's; values near
-//    the ends of the exponent range take the division itself.  Unlike the division's code it has no
-//    slow path for a zero momentum.
+//  * both velocities share the reciprocal of rho: an approximate reciprocal refined by two steps, the
+//    quotient q = m y corrected by its remainder, q' = q - (rho q - m) y.  With y the correctly rounded
+//    reciprocal and an exact remainder, q' is the correctly rounded quotient (Markstein, "Computation of
+//    elementary functions on the IBM RISC System/6000 processor", 1990), that is the IEEE division's,
+//    with its sign also where it is zero (the remainder is then +0, and q - 0 is q).  Divisors and
+//    dividends outside fp64_divisor_ok and fp64_quotient_ok take the division itself.  Unlike the
+//    division's code it has no slow path for a zero momentum.
 //  * U/4 and p's half are exact, so the product and the sum they go into may be fused.
 // 1024^2 step: 160 us with two IEEE divisions and separate products (79 operations a cell without the
 // divisions' own), 147 with the shared reciprocal by three Newton-Raphson steps, 141 with one cubic and
@@ -19,20 +20,32 @@
 
 namespace lbrs {
 
-// The biased exponent lies in [256, 1790]: neither a reciprocal nor a quotient of such numbers, nor a
-// remainder of one, comes near the range's ends.
+// The biased exponent lies in [256, 1790]: the size is between 2^-767 and 2^768.
 __device__ __forceinline__ bool fp64_mid_range(double x)
 {
     const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
     return e - 256u <= 1790u - 256u;
 }
 
-// 1/x, correctly rounded but for a mantissa of all ones (x in the middle range).
+// May x be divided by by its reciprocal?  It is positive and between 2^-250 and 2^251, so that a quotient of
+// a mid-range dividend lies between 2^-1018 and 2^1018 (no overflow, no subnormal) and its remainder, a
+// multiple of 2^-872 at least, is exact.  Not with a mantissa of all ones, whose reciprocal the last step
+// may miss by one unit (1 - 2^-53: 1 instead of 1 + 2^-52).
+__device__ __forceinline__ bool fp64_divisor_ok(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    return (hi >> 20) - 773u <= 500u && (lo & (hi | 0xfff00000u)) != 0xffffffffu;
+}
+
+// 1/x, correctly rounded (fp64_divisor_ok).  The approximation reads and gives the upper word, within
+// 2^-18; the hyperpower step of order three, y (1 + e + e^2) with e = 1 - x y (Altman, "An optimum cubically
+// convergent iterative method of inverting a linear bounded operator in Hilbert space", 1960), leaves
+// e^3 <= 2^-54 and its own rounding, within a unit in the last place; from there a Newton-Raphson step with
+// an exact residual rounds correctly, but for a mantissa of all ones (Markstein).
 __device__ __forceinline__ double fp64_reciprocal(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    // to the cube of the start's error, then one Newton-Raphson step from within a unit in the last place
     const double e = __fma_rn(-x, y, 1.0);
     y = __fma_rn(y, __fma_rn(e, e, e), y);
     return __fma_rn(y, __fma_rn(-x, y, 1.0), y);
@@ -42,7 +55,7 @@ __device__ __forceinline__ double fp64_reciprocal(double x)
 __device__ __forceinline__ double fp64_quotient(double m, double x, double y)
 {
     const double q = m * y;
-    return __fma_rn(__fma_rn(-x, q, m), y, q);
+    return __fma_rn(__fma_rn(x, q, -m), -y, q);
 }
 
 // The test for zero on the integer units: an FP64 comparison costs as much as a product.
@@ -55,11 +68,9 @@ __device__ __forceinline__ bool fp64_quotient_ok(double m)
 struct Fp64Divisor {
     double x, y;
     bool ok;
-    __device__ __forceinline__ explicit Fp64Divisor(double d) : x(d), y(0.0), ok(fp64_mid_range(d))
+    __device__ __forceinline__ explicit Fp64Divisor(double d) : x(d), y(0.0), ok(fp64_divisor_ok(d))
     {
         if (ok) y = fp64_reciprocal(d);
-        // (a mantissa of all ones has no correctly rounded reciprocal here)
-        if (((unsigned)__double2hiint(d) & 0xfffffu) == 0xfffffu && __double2loint(d) == -1) ok = false;
     }
     __device__ __forceinline__ double divide(double m) const
     {
@@ -70,7 +81,7 @@ struct Fp64Divisor {
 template <>
 __device__ __forceinline__ void velocity2<double>(double rho, double mx, double my, double& u, double& v)
 {
-    if (fp64_mid_range(rho) && fp64_quotient_ok(mx) && fp64_quotient_ok(my)) {
+    if (fp64_divisor_ok(rho) && fp64_quotient_ok(mx) && fp64_quotient_ok(my)) {
         const double y = fp64_reciprocal(rho);
         u = fp64_quotient(mx, rho, y);
         v = fp64_quotient(my, rho, y);
@@ -83,7 +94,7 @@ __device__ __forceinline__ void velocity2<double>(double rho, double mx, double 
 template <>
 __device__ __forceinline__ double velocity1<double>(double rho, double m)
 {
-    if (fp64_mid_range(rho) && fp64_quotient_ok(m)) return fp64_quotient(m, rho, fp64_reciprocal(rho));
+    if (fp64_divisor_ok(rho) && fp64_quotient_ok(m)) return fp64_quotient(m, rho, fp64_reciprocal(rho));
     return m / rho;
 }
 
@@ -145,7 +156,7 @@ __device__ __forceinline__ void equilibria1d3<double>(const double U[3], double 
 template <>
 __device__ __forceinline__ double bound_local<double>(const double U[4], double gamma)
 {
-    if (!fp64_mid_range(U[0]) || !fp64_quotient_ok(U[1]) || !fp64_quotient_ok(U[2])) return bound2d<double>(U, gamma);
+    if (!fp64_divisor_ok(U[0]) || !fp64_quotient_ok(U[1]) || !fp64_quotient_ok(U[2])) return bound2d<double>(U, gamma);
     const double gm1 = gamma - 1.0;
     const double y = fp64_reciprocal(U[0]);
     const double u = fp64_quotient(U[1], U[0], y), v = fp64_quotient(U[2], U[0], y);
