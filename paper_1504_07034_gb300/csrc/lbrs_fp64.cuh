@@ -133,7 +133,15 @@ __device__ __forceinline__ void equilibria1d<double>(const double U[3], double g
     }
 }
 
-// U/3 by the reciprocal's product and one correction, as above.
+// U/3 by the reciprocal's product and one correction, as above, at any size: a quotient by three lies at least
+// a sixth of a unit in the last place from a tie, subnormal ones too, and the remainder is exact.  Not for
+// infinities, whose product is the quotient and whose remainder is NaN.
+__device__ __forceinline__ double fp64_third(double m)
+{
+    const double q = fp64_quotient(m, 3.0, 1.0 / 3.0);
+    return ((unsigned)__double2hiint(m) & 0x7ff00000u) == 0x7ff00000u ? m : q;
+}
+
 template <>
 __device__ __forceinline__ void equilibria1d3<double>(const double U[3], double gm1, double c, double e[3][3])
 {
@@ -143,7 +151,7 @@ __device__ __forceinline__ void equilibria1d3<double>(const double U[3], double 
     const double G[3] = {U[1], xx + p, u * (U[2] + p)};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const double a = fp64_quotient(U[k], 3.0, 1.0 / 3.0);
+        const double a = fp64_third(U[k]);
         const double b = c * G[k];
         e[0][k] = a - b;
         e[1][k] = a;

@@ -48,9 +48,11 @@ struct TubeConst {
     P2 c, nc, gm1, ngm1, half, one, third, nthree, om, om1;
 };
 
-// Equilibria of a pair: e[0..2] of the population moving to -x, z of the resting one (Q = 3), r of
-// the one moving to +x.
-template <int Q>
+__device__ __forceinline__ bool tube_ordinary(float q) { return fabsf(q) > 0.f && fabsf(q) < INFINITY; }
+
+// Equilibria of a pair: l[0..2] of the population moving to -x, z of the resting one (Q = 3), r of
+// the one moving to +x.  INF: of infinite moments, too (Q = 3: without it they become NaN).
+template <int Q, bool INF = false>
 __device__ __forceinline__ void tube_feq(const P2 U[3], const TubeConst& m, P2 l[3], P2 z[3], P2 r[3])
 {
     // 1/rho (rcp_f32), with the sign carried along
@@ -69,11 +71,14 @@ __device__ __forceinline__ void tube_feq(const P2 U[3], const TubeConst& m, P2 l
             r[k] = fma2(m.half, U[k], b[k]);
         }
     } else {
-        // U/3 rounded: the reciprocal's product and one correction of the remainder (Markstein)
+        // U/3 rounded: the reciprocal's product and one correction of the remainder (Markstein), at any
+        // size; the product itself is the quotient of a zero (whose sign the correction loses) and of an
+        // infinity (whose remainder is NaN)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const P2 q = mul2(U[k], m.third);
             z[k] = fma2(fma2(q, m.nthree, U[k]), m.third, q);
+            if constexpr (INF) z[k] = pk(tube_ordinary(lo2(q)) ? lo2(z[k]) : lo2(q), tube_ordinary(hi2(q)) ? hi2(z[k]) : hi2(q));
         }
         l[0] = fma2(m.nc, U[1], z[0]);
         r[0] = fma2(m.c, U[1], z[0]);
@@ -92,6 +97,34 @@ struct TubeEnds {
                          // lane's first; -1 elsewhere
     bool any_ghost;      // some lane of the warp has one
 };
+
+// Of a window whose tube begins (first) in lane pad / C and, after g cells of the window, ends (last).
+template <int C>
+__device__ __forceinline__ TubeEnds tube_ends(int lane, int pad, bool first, bool last, int g)
+{
+    TubeEnds w;
+    w.first = first && lane == pad / C;
+    w.last = last && g % C == 0 && lane == g / C - 1;
+    w.ghost = last && lane == g / C && g % C ? g % C : -1;
+    w.any_ghost = last && g % C && g < 32 * C;
+    return w;
+}
+
+__device__ __forceinline__ TubeConst tube_const(const TubeArgs& a, float c)
+{
+    TubeConst m;
+    m.c = pk(c, c);
+    m.nc = pk(-c, -c);
+    m.gm1 = pk(a.gm1, a.gm1);
+    m.ngm1 = pk(-a.gm1, -a.gm1);
+    m.half = pk(0.5f, 0.5f);
+    m.one = pk(1.f, 1.f);
+    m.third = pk(1.f / 3.f, 1.f / 3.f);
+    m.nthree = pk(-3.f, -3.f);
+    m.om = pk(a.om, a.om);
+    m.om1 = pk(a.om1, a.om1);
+    return m;
+}
 
 // Cell j of a lane's C cells kept in pairs (j, j + C/2).
 template <int C>
@@ -205,6 +238,83 @@ __device__ __forceinline__ P2 tube_pair(const float* sm, int lane, int j)
     return pk(sm[lane * (C + 1) + j], sm[lane * (C + 1) + j + C / 2]);
 }
 
+// Some cell of the warp is not finite.  In D1Q3 the steps above turn an infinite moment into NaN, which then
+// stays in its cell's moments and resting population, so that their end shows whether they met one.
+template <int C>
+__device__ __forceinline__ bool tube_not_finite(const P2 (*v)[3])
+{
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < C / 2; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) bad |= !(fabsf(lo2(v[j][k])) < INFINITY) || !(fabsf(hi2(v[j][k])) < INFINITY);
+    return __any_sync(0xffffffffu, bad);
+}
+
+// Where cell x of a tube lies in memory: wrapped, or clamped to its ends.
+__device__ __forceinline__ int64_t tube_place(int64_t off, int len, int periodic, int x)
+{
+    if (periodic) {
+        x %= len;
+        return off + (x < 0 ? x + len : x);
+    }
+    return off + min(max(x, 0), len - 1);
+}
+
+// A window's steps once more with infinities kept (D1Q3), cell by cell in thread-local memory.  Such a state is
+// garbage soon, so this need not be fast.  1024 tubes of 200 to 15000 cells: 16.0 ms without any care, 17.4
+// with it in every step, 15.0 with this call (whose presence also changes the steps' registers, 128 a lane
+// instead of 159); at omega = 1.2, up to 9000 cells: 11.4 without, 12.3 in every step, 11.7 so.
+template <int C>
+__device__ __noinline__ void tube_redo(const TubeArgs& a, float c, bool first, bool last, int64_t off, int len, int x0,
+                                       int ns, int t0, int tlen)
+{
+    const int lane = threadIdx.x & 31, xl = x0 + lane * C;
+    const TubeEnds w = tube_ends<C>(lane, tube_pad<C>(a.halo), first, last, len - x0);
+    const TubeConst m = tube_const(a, c);
+    float f[C][9];                                        // [q * 3 + k]
+#pragma unroll 1
+    for (int j = 0; j < C; ++j) {
+        const int64_t at = tube_place(off, len, a.periodic, xl + j);
+        for (int n = 0; n < 9; ++n) f[j][n] = a.src[LBRS_IX(n * a.N + at, 9 * a.N, 53)];
+    }
+#pragma unroll 1
+    for (int s = 0; s < ns; ++s) {
+        if (w.ghost > 0)
+            for (int k = 0; k < 3; ++k) f[w.ghost][k] = f[w.ghost - 1][k];
+        float right[3], end[3];                           // what the cell before handed on; what follows the lane
+        for (int k = 0; k < 3; ++k) {
+            const float up = __shfl_up_sync(0xffffffffu, f[C - 1][6 + k], 1);
+            const float down = __shfl_down_sync(0xffffffffu, f[0][k], 1);
+            right[k] = w.first ? f[0][6 + k] : up;
+            end[k] = w.last ? f[C - 1][k] : down;
+        }
+#pragma unroll 1
+        for (int j = 0; j < C; ++j) {
+            float g[3][3];
+            P2 U[3], e[3][3];
+            for (int k = 0; k < 3; ++k) {
+                g[0][k] = j + 1 < C ? f[j + 1 < C ? j + 1 : 0][k] : end[k];
+                g[1][k] = f[j][3 + k];
+                g[2][k] = right[k];
+                right[k] = f[j][6 + k];
+                const float u = __fadd_rn(__fadd_rn(g[0][k], g[1][k]), g[2][k]);
+                U[k] = pk(u, u);
+            }
+            tube_feq<3, true>(U, m, e[0], e[1], e[2]);
+            for (int q = 0; q < 3; ++q)
+                for (int k = 0; k < 3; ++k)
+                    f[j][q * 3 + k] = a.om1 == 0.f ? lo2(e[q][k])
+                                                   : lo2(fma2(m.om1, pk(g[q][k], g[q][k]), mul2(m.om, e[q][k])));
+        }
+    }
+#pragma unroll 1
+    for (int j = 0; j < C; ++j) {
+        if (xl + j < t0 || xl + j >= t0 + tlen) continue;
+        for (int n = 0; n < 9; ++n) a.dst[LBRS_IX(n * a.N + off + xl + j, 9 * a.N, 54)] = f[j][n];
+    }
+}
+
 constexpr int kTubeWarps = 4;
 
 // One warp per tile, up to a.halo steps.  UFORM: omega = 1, on the moments.
@@ -242,32 +352,10 @@ __global__ void __launch_bounds__(32 * kTubeWarps) tube_kernel(const __grid_cons
     // they matter to the tile
     const bool first = !a.periodic && t0 == 0, end = !a.periodic && t0 + tlen + a.halo > len;
     const int x0 = end && !first ? len - (WIN - pad) : t0 - pad;
-    TubeEnds w;
-    w.first = first && lane == pad / C;
-    const int g = len - x0;                               // window place of the cell after the last
-    w.last = end && g % C == 0 && lane == g / C - 1;
-    w.ghost = end && lane == g / C && g % C ? g % C : -1;
-    w.any_ghost = end && g % C && g < WIN;
+    const TubeEnds w = tube_ends<C>(lane, pad, first, end, len - x0);
+    const TubeConst m = tube_const(a, c);
 
-    TubeConst m;
-    m.c = pk(c, c);
-    m.nc = pk(-c, -c);
-    m.gm1 = pk(a.gm1, a.gm1);
-    m.ngm1 = pk(-a.gm1, -a.gm1);
-    m.half = pk(0.5f, 0.5f);
-    m.one = pk(1.f, 1.f);
-    m.third = pk(1.f / 3.f, 1.f / 3.f);
-    m.nthree = pk(-3.f, -3.f);
-    m.om = pk(a.om, a.om);
-    m.om1 = pk(a.om1, a.om1);
-
-    auto place = [&](int x) {                             // where cell x lies in memory
-        if (a.periodic) {
-            x %= len;
-            return off + (x < 0 ? x + len : x);
-        }
-        return off + min(max(x, 0), len - 1);
-    };
+    auto place = [&](int x) { return tube_place(off, len, a.periodic, x); };
     auto turn_in = [&](P2(*v)[3]) {
         __syncwarp();
 #pragma unroll
@@ -320,6 +408,8 @@ __global__ void __launch_bounds__(32 * kTubeWarps) tube_kernel(const __grid_cons
         }
         turn_in(U);
         for (int s = 1; s < ns; ++s) tube_step_u<Q, C>(U, m, w);
+        if constexpr (Q == 3)
+            if (tube_not_finite<C>(U)) return tube_redo<C>(a, c, first, end, off, len, x0, ns, t0, tlen);
         P2 v[P][3];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -338,6 +428,8 @@ __global__ void __launch_bounds__(32 * kTubeWarps) tube_kernel(const __grid_cons
         if constexpr (Q == 3) load3(1, Z);
         load3(Q - 1, R);
         for (int s = 0; s < ns; ++s) tube_step_f<Q, C, false>(L, Z, R, m, w);
+        if constexpr (Q == 3)
+            if (tube_not_finite<C>(Z)) return tube_redo<C>(a, c, first, end, off, len, x0, ns, t0, tlen);
         store3(0, L);
         if constexpr (Q == 3) store3(1, Z);
         store3(Q - 1, R);
