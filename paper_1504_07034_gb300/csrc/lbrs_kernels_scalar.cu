@@ -36,15 +36,24 @@ bool scalar_windows_enabled()
     return v != 0;
 }
 
-// A grid that one window holds at four rows a thread (about 5,900 cells) takes all its steps in one
-// launch (64^2: 1.05 us a step; 1.42 with eight rows a thread, 1.33 in 32 x 32 windows of eight steps a
-// launch).  Larger grids: eight steps a launch, windows and rows per thread growing with the grid as
-// the SMs fill (us a step: 256^2 in 64 x 32 windows 1.58, 64 x 64 1.84, 128 x 64 2.88; 512^2 2.13, 1.87,
-// 3.16; 2048^2 17.4, 13.7, and 12.0 in 128 x 64 with eight rows a thread).
+// A grid that one window holds takes all its steps in one launch, up to 6,400 cells (64^2: 1.05 us a step;
+// 1.42 with eight rows a thread, 1.33 in 32 x 32 windows of eight steps a launch.  400 steps: 76^2 in one
+// window 514 us, 84 x 86 631, 125 x 62 605; 96^2 in windows of 64 x 32 568).  Larger grids: eight steps a
+// launch, windows and rows per thread growing with the grid as the SMs fill (us a step: 256^2 in 64 x 32
+// windows 1.58, 64 x 64 1.84, 128 x 64 2.88; 512^2 2.13, 1.87, 3.16; 2048^2 17.4, 13.7, and 12.0 in 128 x 64
+// with eight rows a thread).
+//
+// A window costs its loads and stores whatever the steps, so short calls keep the two-step kernel (us for
+// 2, 3, .. steps by windows and by that kernel: 64^2 17 17 18 and 11 16 20; 76^2 21 21 23 24 and 12 15 19 24;
+// 256^2 13 15 and 11 16; 1024^2 34 36 40 42 44 48 and 17 25 31 39 45 54; 4096^2 230 252 273 296 317 340 and 93
+// 184 184 275 274 365), and so do the last steps of a call that would leave a window mostly unused (4096^2,
+// the last launch of 1, 2, 3, 4 steps 175, 197, 217, 240 by a window and 91, 92, 183, 184 by two steps, beside
+// 30 for distributions to start them from; 2048^2 45, 51, 57, 65 and 31, 31, 62, 62 beside 7).
 ScalarPlan scalar_plan(int nx, int ny, const int bc[4])
 {
+    const int64_t cells = (int64_t)nx * ny;
     ScalarPlan p{};
-    if (bc[0] != BC_PERIODIC && bc[2] != BC_PERIODIC && (int64_t)nx * ny <= 16384) {
+    if (bc[0] != BC_PERIODIC && bc[2] != BC_PERIODIC && cells <= 6400) {
         p.wx = (nx + 3 + 1) / 2 * 2;
         p.wy = ny + 2;
         p.hx = 2;
@@ -53,15 +62,17 @@ ScalarPlan scalar_plan(int nx, int ny, const int bc[4])
         p.ty = ny;
         p.rows = 4;
         p.steps = 512;
+        p.min_steps = cells <= 5200 ? 4 : 5;
         if (threads_for(p.wx, p.wy, p.rows) <= 1024) return p;
     }
-    const int64_t cells = (int64_t)nx * ny;
     p.wx = cells < 1000000 ? 64 : 128;
     p.wy = cells < 150000 ? 32 : 64;
     p.rows = cells < 1000000 ? 4 : 8;
     p.hx = p.hy = p.steps = 8;
     p.tx = p.wx - 16;
     p.ty = p.wy - 16;
+    p.min_steps = cells < 1000000 ? 3 : 7;
+    p.tail = cells < 1000000 ? 0 : (cells < 8000000 ? 2 : 4);
     return p;
 }
 

@@ -186,6 +186,8 @@ struct ScalarPlan {
     int wx, wy, hx, hy, tx, ty;   // window, cells beyond the tile, tile
     int rows;                     // rows a thread owns
     int steps;                    // steps per launch at most
+    int min_steps;                // calls of fewer steps keep the two-step kernel,
+    int tail;                     // as does a last launch of at most so many
 };
 bool scalar_windows_enabled();
 ScalarPlan scalar_plan(int nx, int ny, const int bc[4]);

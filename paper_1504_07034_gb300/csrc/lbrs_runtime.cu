@@ -1177,7 +1177,12 @@ static lbrs_status step_scalar(lbrs_ctx* ctx, int64_t n)
 
 static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
 {
-    if (ctx->splan.steps && n >= 2) return step_scalar(ctx, n);
+    if (ctx->splan.steps && n >= ctx->splan.min_steps) {
+        const int64_t w = ctx->splan.steps, last = n > w + 1 ? (n - 1) % w : 0, tail = last <= ctx->splan.tail ? last : 0;
+        lbrs_status st = step_scalar(ctx, n - tail);
+        if (st != LBRS_OK || !tail) return st;
+        n = tail;                                  // by the two-step kernel, below
+    }
     if (blocked_1d(ctx)) {
         for (int64_t left = n; left > 0;) {
             const int m = (int)(left < kOneHalo ? left : kOneHalo);

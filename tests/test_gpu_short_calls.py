@@ -1,0 +1,97 @@
+"""Calls of few steps: a kernel of many steps a launch must not take a call that the kernel it replaced does
+faster.  Each case is timed with the default choice and with the switch that turns the many-step kernel off
+(the least of repeated calls on warm caches, launches queued behind a waiting kernel so that the host's time
+is not in it): the default may not take more than 12 % and 1.5 us longer.  The states must agree bit for bit."""
+import json
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+_SCRIPT = r"""
+import json, sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np, torch
+from paper_1504_07034_gb300.solver import Solver
+
+T, P = ("transmissive", None), ("periodic", None)
+D = lambda a, b: ("dirichlet", (a, b, 0.0, 0.0))
+
+
+def best(fn):
+    for _ in range(3):
+        fn()
+    ts = []
+    for _ in range(25):
+        torch.cuda._sleep(400000)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        torch.cuda.synchronize()
+        ts.append(1e3 * a.elapsed_time(b))
+    return min(ts)
+
+
+def solver(c):
+    nx, ny = c["nx"], c["ny"]
+    x, y = torch.arange(nx, device="cuda") / nx, torch.arange(ny, device="cuda") / ny
+    if c["kind"] == "scalar":
+        s = Solver("d2q4s", nx, ny, lam=2.6, dx=1.0 / nx, bc=[D(1.0, 0.0), D(-1.0, 0.2), D(1.0, -2.0), T], precision="f32")
+        return s, (torch.cos(7 * x)[None, :] * torch.sin(5 * y)[:, None] + 0.1)[None].double()
+    s = Solver("d2q4", nx, ny, lam=5.0, dx=1.0 / ny, bc=[P] * 4 if c.get("periodic") else [T] * 4,
+               omega=c.get("omega", 1.0), precision="f32")
+    if c["kind"] == "walls":
+        solid = torch.zeros(ny, nx, dtype=torch.uint8)
+        solid[:ny // 5, nx // 5:] = 1
+        s.set_obstacles(solid)
+    w = 0.1 * torch.cos(6.2831853 * x)[None, :] * torch.sin(6.2831853 * y)[:, None]
+    return s, torch.stack([1.0 + w, 0.3 + w, 0.2 - w, 1.0 - w]).double()
+
+
+times, states = [], []
+for c in json.loads(sys.argv[2]):
+    s, W = solver(c)
+    n = c["n"]
+    hist = s._fields_tensor(n) if c.get("record") else None
+    run = (lambda: s.step_record(n, hist)) if c.get("record") else (lambda: s.step(n))
+    s.set_state(W)
+    run()
+    states.append(s.raw_state().cpu().numpy())
+    if c.get("record"):
+        states.append(hist.cpu().numpy().view(np.uint8).ravel())
+    times.append(best(run))
+    s.close()
+np.savez(sys.argv[3], times=np.array(times), **{f"s{k}": v for k, v in enumerate(states)})
+"""
+
+
+def _compare(tmp_path, cases, off):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    script = tmp_path / "short.py"
+    script.write_text(_SCRIPT)
+    res = {}
+    for name, env in (("default", {}), ("off", off)):
+        out = tmp_path / f"{name}.npz"
+        subprocess.run([sys.executable, str(script), root, json.dumps(cases), str(out)], check=True,
+                       env=dict(os.environ, **env), timeout=600)
+        res[name] = np.load(out)
+    for k in res["off"].files:
+        if k != "times":
+            assert np.array_equal(res["default"][k], res["off"][k]), k
+    slow = [(c, round(a, 1), round(b, 1)) for c, a, b in zip(cases, res["default"]["times"], res["off"]["times"])
+            if a > 1.12 * b + 1.5]
+    assert not slow, slow
+
+
+def test_scalar_windows(tmp_path):
+    """One window, windows of either size, and calls that leave a short rest after full windows."""
+    sizes = [(64, 64, (2, 3, 4)), (80, 80, (2, 3, 4, 5)), (125, 62, (2, 3, 4)), (256, 250, (2, 3)), (768, 768, (2, 3)),
+             (1024, 1000, (2, 3, 4, 5, 6, 7, 10)), (2048, 2048, (2, 4, 6, 10, 11)), (3000, 3000, (2, 3, 4, 6, 10, 12, 13, 18)),
+             (4096, 4090, (2, 4, 6, 10, 11, 12, 18))]
+    _compare(tmp_path, [{"kind": "scalar", "nx": nx, "ny": ny, "n": n} for nx, ny, ns in sizes for n in ns],
+             {"LBRS_F32S_WINDOW": "0"})
