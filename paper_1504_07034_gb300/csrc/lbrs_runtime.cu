@@ -456,8 +456,16 @@ cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int 
 
 // Distribution storage enters and leaves the moments once per call (80 + 80 B per cell, two
 // launches): worth it from this many steps on (1024^2: 6 steps in 45 us instead of 80 us; 128^2:
-// 8 steps in 37 us instead of 41, 6 in 33 instead of 30).
-int64_t march_min(const lbrs_ctx* ctx) { return ctx->N < 400000 ? 8 : 6; }
+// 8 steps in 37 us instead of 41, 6 in 33 instead of 30).  With internal walls an even call takes a
+// storing step beside (step_march), worth it later as the traffic of the three grows beside the pairs'
+// (us on the moments and by storing steps, 1800 x 600 6 steps 128 and 122; 2400 x 800 6, 8 steps 210 and 167,
+// 245 and 222; 2048 x 1024 10 steps 304 and 290; 4096 x 1024 10, 12 steps 571 and 516, 647 and 618).
+int64_t march_min(const lbrs_ctx* ctx, int64_t n)
+{
+    if (ctx->solid && n % 2 == 0 && ctx->N >= 1000000)
+        return ctx->N < 1500000 ? 8 : (ctx->N < 2000000 ? 10 : (ctx->N < 4000000 ? 12 : 14));
+    return ctx->N < 400000 ? 8 : 6;
+}
 
 // Steps the next launch takes out of `left`: three where the three-step kernel applies (but
 // 2 + 2 rather than 3 + 1), else two where the two-step kernel does, else one.  Beside the marching
@@ -785,7 +793,7 @@ cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U, const uint8_t* 
 lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
 {
     const size_t stride = (size_t)ctx->K * ctx->N * elem_bytes(ctx);
-    if (march(ctx) && n >= march_min(ctx)) {
+    if (march(ctx) && n >= march_min(ctx, n)) {
         LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], U_hist));
         lbrs_status st = record_march(ctx, U_hist, n - 1, U_hist + stride);
         if (st != LBRS_OK) return st;
@@ -1207,7 +1215,7 @@ static lbrs_status step_plain(lbrs_ctx* ctx, int64_t n)
     }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBRS_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cap));
-    if (on_moments(ctx) && (ctx->f32u || n >= march_min(ctx))) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
+    if (on_moments(ctx) && (ctx->f32u || n >= march_min(ctx, n))) return step_march(ctx, n, cap == cudaStreamCaptureStatusNone);
     int64_t left = n;
     const int G = graph_steps(ctx);
     if (cap == cudaStreamCaptureStatusNone && n >= 2 * G) {

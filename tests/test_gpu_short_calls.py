@@ -95,3 +95,11 @@ def test_scalar_windows(tmp_path):
              (4096, 4090, (2, 4, 6, 10, 11, 12, 18))]
     _compare(tmp_path, [{"kind": "scalar", "nx": nx, "ny": ny, "n": n} for nx, ny, ns in sizes for n in ns],
              {"LBRS_F32S_WINDOW": "0"})
+
+
+def test_internal_walls_on_the_moments(tmp_path):
+    """Even calls take a storing step before the pairs."""
+    sizes = [(960, 320, (6, 7, 8)), (1800, 600, (6, 8)), (2400, 800, (6, 8, 10)), (2048, 1024, (6, 7, 8, 10, 12)),
+             (4096, 1024, (6, 8, 10, 12, 14))]
+    _compare(tmp_path, [{"kind": "walls", "nx": nx, "ny": ny, "n": n} for nx, ny, ns in sizes for n in ns],
+             {"LBRS_F32_MARCH": "0"})
