@@ -203,12 +203,23 @@ static int fmarch_rows(int nx, int ny)
     return n > 12 ? 8 : (int)std::max<int64_t>(n, 1);
 }
 
-// The marching kernel rather than three steps a launch on tiles?  While one wave takes at most 10 rows, up to
-// about a million cells, whose two buffers the second-level cache holds in good part (us per step, periodic,
-// tiles against march: 128^2 3.23, 1.58; 400^2 4.30, 2.76; 800^2 8.3, 6.3; 1000^2 12.3, 11.6; 1200^2 15.9,
-// 17.9; 2048^2 37, 50).  Grids that the tiles' tensor copies cannot take march at any size (2047^2: two steps
-// on tiles by plain loads 57.8, march 52.0).
-bool fmarch_beats_tiles(int nx, int ny) { return fmarch_wave_rows(nx, ny) <= 10; }
+// The marching kernel rather than the tile kernel's two steps a launch?  While one wave takes at most 10 rows
+// (1024^2, calls of two: 30.8 us against 34.8, recording 38.9 against 43.0).  Grids that the tiles' tensor
+// copies cannot take march at any size (2047^2: two steps on tiles by plain loads 57.8 us a step, march 52.0).
+bool fmarch_beats_pairs(int nx, int ny) { return fmarch_wave_rows(nx, ny) <= 10; }
+
+// Rather than three steps a launch on tiles?  Up to about a million cells, whose two buffers the second-level
+// cache holds in good part (us per step, periodic, tiles against march: 128^2 3.99, 2.91; 512^2 6.19, 5.21;
+// 800^2 9.07, 7.41; 960^2 12.1, 11.5; 1000^2 13.35, 12.65; 1008^2 13.4, 13.1; 2048 x 500 12.9, 13.1; 1024^2 13.2,
+// 13.4; 2048^2 37, 50).  The march has no work beside sides of other kinds where the tiles do (clamped, 1024^2
+// 14.5, 13.5).  Recording adds 32 B a cell to every two steps of either, which costs the march more (800^2
+// 10.4, 10.3; 896^2 12.5, 13.5; 1024^2 15.1, 17.8).
+bool fmarch_beats_threes(int nx, int ny, bool periodic, bool record)
+{
+    const int64_t rows = fmarch_wave_rows(nx, ny);
+    if (record) return rows <= 6;
+    return rows <= 10 && (!periodic || (int64_t)nx * ny <= 1020000);
+}
 
 cudaError_t launch_fmarch_f32(const StepArgs<float>& s, const float ghost[4][GHOST_STRIDE], bool chained,
                               cudaStream_t st)

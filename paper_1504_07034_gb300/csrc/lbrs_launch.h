@@ -268,7 +268,10 @@ bool adapt_moments_enabled();
 cudaError_t launch_fmarch_f32(const StepArgs<float>& a, const float ghost[4][GHOST_STRIDE], bool chained,
                               cudaStream_t s);
 bool fmarch_enabled();
-bool fmarch_beats_tiles(int nx, int ny);
+// The marching kernel rather than the tiles' two-step kernel, or than three steps a launch on tiles
+// (periodic: all sides; record: recording steps)?
+bool fmarch_beats_pairs(int nx, int ny);
+bool fmarch_beats_threes(int nx, int ny, bool periodic, bool record);
 cudaError_t launch_set_state_f32u(const void* W, int w_dtype, int kind, void* fs, int64_t N, int64_t plane,
                                   double gamma, cudaStream_t s);
 // U = U(W) in FP32, g = 0, then the per-field scales from max |U_k| (absmax_bits: 4 words of scratch).

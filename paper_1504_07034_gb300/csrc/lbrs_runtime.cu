@@ -396,10 +396,16 @@ bool fmarch(const lbrs_ctx* ctx)
     if (ctx->ny_store > kMaxGridY) return false;
     if (!fmarch_enabled() || !fused2_f32(ctx) || !step3_f32_enabled() || ctx->solid || ctx->cfg.omega == 1.0) return false;
     if (ctx->cfg.bc[2].kind == LBRS_BC_WALL_HALFWAY || ctx->cfg.bc[3].kind == LBRS_BC_WALL_HALFWAY) return false;
-    return !step3_tiles(ctx) || fmarch_beats_tiles((int)ctx->cfg.nx, (int)ctx->ny_store);
+    return !step3_tiles(ctx) || fmarch_beats_pairs((int)ctx->cfg.nx, (int)ctx->ny_store);
 }
 
-bool fused3(const lbrs_ctx* ctx) { return step3_tiles(ctx) && !fmarch(ctx); }
+// Three steps a launch on tiles as long as three are left?  (record: recording steps.)
+bool fused3(const lbrs_ctx* ctx, bool record = false)
+{
+    if (!step3_tiles(ctx)) return false;
+    const bool periodic = ctx->cfg.bc[0].kind == LBRS_BC_PERIODIC && ctx->cfg.bc[2].kind == LBRS_BC_PERIODIC;
+    return !fmarch(ctx) || !fmarch_beats_threes((int)ctx->cfg.nx, (int)ctx->ny_store, periodic, record);
+}
 
 // FP32 at omega = 1 (distributions or moments-only storage) on the moments by the marching kernel
 // (lbrs_march.cuh), two steps a launch?  Not with halfway walls; the switches that ask for one, two
@@ -801,7 +807,7 @@ lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
         return LBRS_OK;
     }
     int64_t m = 0;
-    for (; m + 3 <= n && n - m != 4 && fused3(ctx); m += 3) {
+    for (; m + 3 <= n && n - m != 4 && fused3(ctx, true); m += 3) {
         LBRS_CUDA(ctx, launch_record_step3(ctx, U_hist + m * stride));
         ctx->cur ^= 1;
         ctx->launches += 1;

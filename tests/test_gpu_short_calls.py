@@ -103,3 +103,15 @@ def test_internal_walls_on_the_moments(tmp_path):
              (4096, 1024, (6, 8, 10, 12, 14))]
     _compare(tmp_path, [{"kind": "walls", "nx": nx, "ny": ny, "n": n} for nx, ny, ns in sizes for n in ns],
              {"LBRS_F32_MARCH": "0"})
+
+
+def test_full_collision_march(tmp_path):
+    """omega != 1: the marching kernel, three steps a launch on tiles and pairs beside them, recording and not,
+    on either side of the rules' lines."""
+    plain = [(128, 128, (2, 4, 8)), (800, 800, (2, 4, 6, 8)), (1024, 1024, (2, 4, 5, 6, 12, 24)), (2048, 500, (6, 12))]
+    record = [(128, 128, (2, 4, 6)), (800, 800, (2, 6, 12)), (896, 896, (2, 6, 12)), (1024, 1024, (2, 4, 5, 6, 8, 12)),
+              (4096, 250, (6, 9))]
+    cases = [{"kind": "euler", "periodic": True, "omega": 1.5, "nx": nx, "ny": ny, "n": n, "record": r}
+             for r, sizes in ((False, plain), (True, record)) for nx, ny, ns in sizes for n in ns]
+    cases += [{"kind": "euler", "omega": 1.5, "nx": 1024, "ny": 1024, "n": n} for n in (2, 6, 12)]
+    _compare(tmp_path, cases, {"LBRS_F32_FMARCH": "0"})
