@@ -8,8 +8,10 @@
 // covers the first active_tiles(L) tiles with up to H steps each
 // (temporal blocking, lbrs_batch.cuh).  Tubes whose last launch left them in
 // the other buffer are copied back by one final kernel.  The launch sequence
-// of a run is captured once into a CUDA graph and replayed while the steps
-// and the tuning stay the same.  An autotuner times one launch of each
+// of a run is captured once from either buffer into a CUDA graph and replayed
+// while the steps and the tuning stay the same (512 tubes of 1000 cells, one
+// launch of 17 steps: 24 us; 57 when a state in the other buffer meant a new
+// plan).  An autotuner times one launch of each
 // candidate (block size, cells per thread, H) on the current state and keeps
 // the fastest per lattice update.
 #include <math.h>
@@ -100,12 +102,13 @@ struct lbrs_batch {
     cudaStream_t stream;
     lbrs_batch_tuning tuning;
     int64_t launches;
-    // cached plan and graph of the last run
+    // plan of the last run, whose tables are on the device (valid while plan_steps is not empty), and its
+    // graphs from either buffer: an odd number of launches leaves the state in the other one
     std::vector<int64_t> plan_steps;
     lbrs_batch_tuning plan_tuning;
-    int plan_cur;
-    int plan_nlaunch;
-    cudaGraphExec_t graph;
+    std::vector<int> plan_active;
+    int plan_nlaunch, plan_ncopy;
+    cudaGraphExec_t graph[2];
     cudaStream_t cap_stream;
     char err[512];
 };
@@ -249,21 +252,28 @@ cudaError_t launch_one(lbrs_batch* B, int from, const lbrs_batch_tuning& t, int 
     return launch_batch_f32(batch_args<float>(B, from, t, launch), ntiles, t.block, s);
 }
 
+void drop_graphs(lbrs_batch* B)
+{
+    for (cudaGraphExec_t& g : B->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 // Upload the tube steps and the tile tables of a run; returns the launch plan.
 lbrs_status upload_plan(lbrs_batch* B, const int64_t* steps, const lbrs_batch_tuning& t, std::vector<int>& active,
-                        int& nlaunch, int& ncopy, int& final_parity)
+                        int& nlaunch, int& ncopy)
 {
     std::vector<BatchTile> tiles;
     plan(B, steps, t, tiles, active, nlaunch);
     if ((int64_t)tiles.size() > B->L.max_tiles) return bfail(B, LBRS_EINVAL, "tile table overflow");
     std::vector<int> st(B->cfg.batch);
     for (int64_t b = 0; b < B->cfg.batch; ++b) st[b] = (int)steps[b];
-    final_parity = (B->cur + nlaunch) & 1;
-    // tubes whose last launch left them in the other buffer
+    // tubes whose last launch left them in another buffer than the run's last one
     std::vector<BatchTile> copies;
     for (int64_t b = 0; b < B->cfg.batch; ++b) {
         const int64_t nl = (steps[b] + t.halo - 1) / t.halo;
-        if (((B->cur + nl) & 1) != final_parity)
+        if ((nl ^ nlaunch) & 1)
             for (int64_t x = 0; x < B->lengths[b]; x += 4096)
                 copies.push_back(BatchTile{(int)b, (int)x, (int)std::min<int64_t>(4096, B->lengths[b] - x), 0});
     }
@@ -383,7 +393,7 @@ lbrs_status lbrs_batch_create(const lbrs_batch_config* cfg, void* d_workspace, s
 void lbrs_batch_destroy(lbrs_batch* B)
 {
     if (!B) return;
-    if (B->graph) cudaGraphExecDestroy(B->graph);
+    drop_graphs(B);
     if (B->cap_stream) cudaStreamDestroy(B->cap_stream);
     delete B;
 }
@@ -441,28 +451,26 @@ lbrs_status lbrs_batch_run(lbrs_batch* B, const int64_t* steps)
         max_steps = std::max(max_steps, steps[b]);
     }
     if (max_steps == 0) return LBRS_OK;
-    const lbrs_batch_tuning t = B->tuning;
-    const bool same = B->graph && B->plan_cur == B->cur && !memcmp(&B->plan_tuning, &t, sizeof t) &&
-                      B->plan_steps.size() == (size_t)B->cfg.batch &&
+    lbrs_batch_tuning t = B->tuning;
+    // in registers the tiles follow from the halo: no more of it than there are steps
+    if (in_registers(B, t)) t.halo = (int)std::min<int64_t>(t.halo, max_steps);
+    const bool same = !memcmp(&B->plan_tuning, &t, sizeof t) && B->plan_steps.size() == (size_t)B->cfg.batch &&
                       std::equal(B->plan_steps.begin(), B->plan_steps.end(), steps);
-    int final_parity;
-    if (same) {
-        BCUDA(B, cudaGraphLaunch(B->graph, B->stream));
-        final_parity = (B->cur + B->plan_nlaunch) & 1;
-        B->launches += B->plan_nlaunch + 1;
-    } else {
-        std::vector<int> active;
-        int nlaunch, ncopy;
-        lbrs_status st = upload_plan(B, steps, t, active, nlaunch, ncopy, final_parity);
+    if (!same) {
+        B->plan_steps.clear();
+        lbrs_status st = upload_plan(B, steps, t, B->plan_active, B->plan_nlaunch, B->plan_ncopy);
         if (st != LBRS_OK) return st;
-        if (B->graph) {
-            cudaGraphExecDestroy(B->graph);
-            B->graph = nullptr;
-        }
+        drop_graphs(B);               // (the upload has waited for their last run)
+        B->plan_tuning = t;
+        B->plan_steps.assign(steps, steps + B->cfg.batch);
+    }
+    const int final_parity = (B->cur + B->plan_nlaunch) & 1;
+    cudaGraphExec_t& graph = B->graph[B->cur];
+    if (!graph) {
         if (!B->cap_stream) BCUDA(B, cudaStreamCreateWithFlags(&B->cap_stream, cudaStreamNonBlocking));
         BCUDA(B, prepare(B, t));
         BCUDA(B, cudaStreamBeginCapture(B->cap_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t le = enqueue_run(B, t, active, nlaunch, ncopy, final_parity, B->cap_stream);
+        cudaError_t le = enqueue_run(B, t, B->plan_active, B->plan_nlaunch, B->plan_ncopy, final_parity, B->cap_stream);
         cudaGraph_t g = nullptr;
         cudaError_t ee = cudaStreamEndCapture(B->cap_stream, &g);
         if (le != cudaSuccess || ee != cudaSuccess) {
@@ -470,19 +478,15 @@ lbrs_status lbrs_batch_run(lbrs_batch* B, const int64_t* steps)
             return bfail(B, LBRS_ECUDA, "capturing the run: %s",
                          cudaGetErrorString(le != cudaSuccess ? le : ee));
         }
-        cudaError_t ie = cudaGraphInstantiate(&B->graph, g, 0);
+        cudaError_t ie = cudaGraphInstantiate(&graph, g, 0);
         cudaGraphDestroy(g);
         if (ie != cudaSuccess) {
-            B->graph = nullptr;
+            graph = nullptr;
             return bfail(B, LBRS_ECUDA, "instantiating the run graph: %s", cudaGetErrorString(ie));
         }
-        B->plan_steps.assign(steps, steps + B->cfg.batch);
-        B->plan_tuning = t;
-        B->plan_cur = B->cur;
-        B->plan_nlaunch = nlaunch;
-        BCUDA(B, cudaGraphLaunch(B->graph, B->stream));
-        B->launches += nlaunch + (ncopy > 0);
     }
+    BCUDA(B, cudaGraphLaunch(graph, B->stream));
+    B->launches += B->plan_nlaunch + (B->plan_ncopy > 0);
     B->cur = final_parity;
     return LBRS_OK;
 }
@@ -498,6 +502,7 @@ lbrs_status lbrs_batch_autotune(lbrs_batch* B, const int64_t* steps, lbrs_batch_
     cudaEvent_t e0, e1;
     BCUDA(B, cudaEventCreate(&e0));
     BCUDA(B, cudaEventCreate(&e1));
+    B->plan_steps.clear();        // the candidates' plans take the tables
     double best = 1e300;
     lbrs_batch_tuning best_t = B->tuning;
     lbrs_status result = LBRS_OK;
@@ -509,8 +514,8 @@ lbrs_status lbrs_batch_autotune(lbrs_batch* B, const int64_t* steps, lbrs_batch_
                 if (in_registers(B, t) && (bi != 256 || ci != 4)) continue;   // the halo alone matters there
                 if (prepare(B, t) != cudaSuccess) continue;
                 std::vector<int> active;
-                int nlaunch, ncopy, fp;
-                lbrs_status st = upload_plan(B, steps, t, active, nlaunch, ncopy, fp);
+                int nlaunch, ncopy;
+                lbrs_status st = upload_plan(B, steps, t, active, nlaunch, ncopy);
                 if (st != LBRS_OK) {
                     result = st;
                     break;
@@ -539,10 +544,6 @@ lbrs_status lbrs_batch_autotune(lbrs_batch* B, const int64_t* steps, lbrs_batch_
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (result != LBRS_OK) return result;
-    if (B->graph) {               // the tile table now holds the last candidate's plan
-        cudaGraphExecDestroy(B->graph);
-        B->graph = nullptr;
-    }
     B->tuning = best_t;
     if (chosen) *chosen = best_t;
     if (ns_per_update) *ns_per_update = best;

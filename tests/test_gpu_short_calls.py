@@ -115,3 +115,57 @@ def test_full_collision_march(tmp_path):
              for r, sizes in ((False, plain), (True, record)) for nx, ny, ns in sizes for n in ns]
     cases += [{"kind": "euler", "omega": 1.5, "nx": 1024, "ny": 1024, "n": n} for n in (2, 6, 12)]
     _compare(tmp_path, cases, {"LBRS_F32_FMARCH": "0"})
+
+
+def test_repeated_batch_runs():
+    """Runs of one launch leave the state in the other buffer each time: repeating one must not take longer than
+    repeating a run of two launches (both replay what the first runs planned).  Any sequence of runs, plans and
+    tunings equals one run of all steps bit for bit."""
+    import time
+
+    import torch
+    from paper_1504_07034_gb300.solver import BatchSolver
+
+    def batch(lengths, lattice, omega):
+        b = BatchSolver(lengths, [4.0] * len(lengths), precision="f32", lattice=lattice, omega=omega)
+        x = torch.arange(int(sum(lengths)), device="cuda").double()
+        b.set_state(torch.stack([1.0 + 0.1 * torch.cos(x / 7), 0.1 * torch.sin(x / 5), 1.0 - 0.1 * torch.sin(x / 11)]))
+        return b
+
+    b = batch([200] * 8, "d1q2", 1.0)
+
+    def seconds(n, reps=40):
+        steps = np.full(8, n)
+        for _ in range(4):
+            b.run(steps)
+        torch.cuda.synchronize()
+        best = np.inf
+        for _ in range(5):
+            t = time.perf_counter()
+            for _ in range(reps):
+                b.run(steps)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        return best / reps
+
+    one, two = seconds(17), seconds(40)
+    b.close()
+    assert one < 1.1 * two, (one, two)
+
+    lengths = [1, 5, 33, 64, 65, 200, 449, 1000]
+    for lattice, omega in (("d1q2", 1.0), ("d1q2", 1.3), ("d1q3", 1.0), ("d1q3", 0.9)):
+        a, c = batch(lengths, lattice, omega), batch(lengths, lattice, omega)
+        total = np.zeros(len(lengths), dtype=np.int64)
+        uneven = np.array([17, 3, 40, 0, 1, 33, 64, 5])
+        for k, steps in enumerate((1, 1, 2, 17, 17, 40, 40, uneven, uneven, 17, 31, 32, 33, uneven, 5)):
+            steps = np.broadcast_to(steps, total.shape).astype(np.int64)
+            a.run(steps)
+            total += steps
+            if k == 8:
+                a.autotune(steps)
+                a.tuning = (256, 4, 32)
+        c.tuning = (256, 2, 128)              # the shared-memory kernel
+        c.run(total)
+        assert torch.equal(a.get_distributions(), c.get_distributions()), (lattice, omega)
+        a.close()
+        c.close()
