@@ -182,7 +182,7 @@ size_t smem_of(const lbrs_batch* B, const lbrs_batch_tuning& t)
 cudaError_t prepare(const lbrs_batch* B, const lbrs_batch_tuning& t)
 {
     if (in_registers(B, t)) return cudaSuccess;
-    return B->f64 ? prepare_batch_f64(t.block, smem_of(B, t), B->q) : prepare_batch_f32(t.block, smem_of(B, t), B->q);
+    return B->f64 ? prepare_batch_f64(t.block, B->q) : prepare_batch_f32(t.block, B->q);
 }
 
 // Tubes ordered by decreasing steps (stable) and their tiles in that order.

@@ -2130,24 +2130,26 @@ cudaError_t launch_batch_f32(const BatchArgs<float>& a, int ntiles, int block, c
 }
 
 template <int Q>
-static cudaError_t prepare_batch_q_f32(int block, size_t smem)
+static cudaError_t prepare_batch_q_f32(int block)
 {
-    // opt in to more than the default 48 KiB of dynamic shared memory
+    // opt in to more than the default 48 KiB of dynamic shared memory: to all there is, so that no launch
+    // shape lowers the limit of another
+    constexpr int smem = 227 * 1024;
     switch (block) {
         case 128:
-            return cudaFuncSetAttribute(batch1d_kernel<float, 128, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<float, 128, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         case 256:
-            return cudaFuncSetAttribute(batch1d_kernel<float, 256, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<float, 256, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         case 512:
-            return cudaFuncSetAttribute(batch1d_kernel<float, 512, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<float, 512, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         default:
             return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t prepare_batch_f32(int block, size_t smem, int q)
+cudaError_t prepare_batch_f32(int block, int q)
 {
-    return q == 3 ? prepare_batch_q_f32<3>(block, smem) : prepare_batch_q_f32<2>(block, smem);
+    return q == 3 ? prepare_batch_q_f32<3>(block) : prepare_batch_q_f32<2>(block);
 }
 
 cudaError_t launch_batch_copy_f32(const float* src, float* dst, int64_t N, const BatchTile* tiles, int ntiles,

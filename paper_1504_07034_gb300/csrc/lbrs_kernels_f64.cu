@@ -826,24 +826,26 @@ cudaError_t launch_batch_f64(const BatchArgs<double>& a, int ntiles, int block, 
 }
 
 template <int Q>
-static cudaError_t prepare_batch_q_f64(int block, size_t smem)
+static cudaError_t prepare_batch_q_f64(int block)
 {
-    // opt in to more than the default 48 KiB of dynamic shared memory
+    // opt in to more than the default 48 KiB of dynamic shared memory: to all there is, so that no launch
+    // shape lowers the limit of another
+    constexpr int smem = 227 * 1024;
     switch (block) {
         case 128:
-            return cudaFuncSetAttribute(batch1d_kernel<double, 128, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<double, 128, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         case 256:
-            return cudaFuncSetAttribute(batch1d_kernel<double, 256, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<double, 256, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         case 512:
-            return cudaFuncSetAttribute(batch1d_kernel<double, 512, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(batch1d_kernel<double, 512, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         default:
             return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t prepare_batch_f64(int block, size_t smem, int q)
+cudaError_t prepare_batch_f64(int block, int q)
 {
-    return q == 3 ? prepare_batch_q_f64<3>(block, smem) : prepare_batch_q_f64<2>(block, smem);
+    return q == 3 ? prepare_batch_q_f64<3>(block) : prepare_batch_q_f64<2>(block);
 }
 
 cudaError_t launch_batch_copy_f64(const double* src, double* dst, int64_t N, const BatchTile* tiles, int ntiles,

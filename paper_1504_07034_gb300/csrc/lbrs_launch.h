@@ -214,8 +214,8 @@ cudaError_t launch_tube_f64(int q, const StepArgs<double>& a, int steps, cudaStr
 cudaError_t launch_batch_f64(const BatchArgs<double>& a, int ntiles, int block, cudaStream_t s);
 cudaError_t launch_batch_f32(const BatchArgs<float>& a, int ntiles, int block, cudaStream_t s);
 // Raise the kernel's dynamic shared-memory limit to smem bytes (call before launching or capturing).
-cudaError_t prepare_batch_f64(int block, size_t smem, int q);
-cudaError_t prepare_batch_f32(int block, size_t smem, int q);
+cudaError_t prepare_batch_f64(int block, int q);
+cudaError_t prepare_batch_f32(int block, int q);
 cudaError_t launch_batch_copy_f64(const double* src, double* dst, int64_t N, const BatchTile* tiles, int ntiles,
                                   const int64_t* tube_off, int planes, cudaStream_t s);
 cudaError_t launch_batch_copy_f32(const float* src, float* dst, int64_t N, const BatchTile* tiles, int ntiles,

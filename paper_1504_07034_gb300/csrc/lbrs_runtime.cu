@@ -307,8 +307,8 @@ cudaError_t launch_one_step(lbrs_ctx* ctx, int from, cudaStream_t s)
 }
 
 // FP32 1-D (D1Q2, D1Q3) with both ends transmissive or both periodic: up to kOneHalo steps per launch
-// by the tubes' register kernel (lbrs_tube.cuh; the single-tube arithmetic, bit-identical to one step
-// a launch).  LBRS_1D_BLOCKED=0 keeps one step a launch.
+// by the tubes' kernels in registers or shared memory (launch_one_tube_f32; the single-tube arithmetic,
+// bit-identical to one step a launch).  LBRS_1D_BLOCKED=0 keeps one step a launch.
 constexpr int kOneHalo = 32;
 
 bool blocked_1d_enabled()
