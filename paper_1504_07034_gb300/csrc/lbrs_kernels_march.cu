@@ -183,8 +183,10 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
 }
 
 // Time of an iteration (K source rows) with w warps per SM sub-partition, in us (periodic, K = 2: 768^2
-// 0.34 at one on the fullest, 900^2 0.44 at two, 2048 x 512 0.63 at three, 1200^2 0.81 at four, 1.02 at
-// five), full waves and a rest beyond.
+// 0.34 at one on the fullest, 900^2 0.44 at two, 2048 x 512 0.63 at three, 1200^2 0.81 at four), full waves and
+// a rest beyond.  A wave of one more warp measured 0.22 on top; taken as 0.32, because the rest starts late:
+// with 0.22 the rule picks 38 rows instead of 42 at 2400^2 (26.7 us a step instead of 21.0) and 64 instead of
+// 50 at 6144 x 2048 (49.1 instead of 44.7).
 double march_iteration(double w)
 {
     static const double t[5] = {0.34, 0.34, 0.44, 0.63, 0.80};
@@ -263,9 +265,10 @@ bool march_enabled() { return march_mode() != 0; }
 // The tile kernel's two-step launch (step2d_u2_kernel, 32 x 16 tiles, four blocks per SM) starts
 // faster than a march and wins on small grids: about 2.7 us and 1.05 us per tile of an SM against the
 // march's 1.5 us and its iterations, 1 us and a quarter more of them beside sides that are not periodic
-// (per launch, in a graph: 128^2 3.7 against 4.4 us periodic and 5.4 with clamped sides, 384^2 4.5 against 5.6 and
-// 6.5, 512^2 6.7 against 5.6 and 6.6, 1531 x 200 6.9 against 6.4 and 10.0, 768^2 10.7 against 7.9 and
-// 8.8).
+// (us per launch, in a graph, tiles and march, periodic and then with clamped sides: 128^2 3.1, 4.1 and 2.9, 4.9;
+// 256^2 3.1, 5.1 and 3.0, 6.0; 384^2 4.4, 4.9 and 4.2, 6.9; 448^2 5.1, 4.9 and 5.0, 6.9; 512^2 6.4, 5.0 and 6.2,
+// 6.3; 1531 x 200 6.7, 5.9 and 6.7, 8.5; 640^2 8.4, 5.9 and 8.2, 6.8; 768^2 10.3, 7.6 and 10.2, 7.8.  Of 54 grids
+// and side sets from 64^2 to 1531 x 973 the choice is at most 4 % slower than the other kernel.)
 bool march_prefers_tiles(int nx, int ny, const int bc[4])
 {
     if (march_mode() >= 2) return false;
