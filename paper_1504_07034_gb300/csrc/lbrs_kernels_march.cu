@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
     const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= N) return;
     const bool two = i + 1 < N;
-    const bool keep0 = solid && solid[i], keep1 = !two || (solid && solid[two ? i + 1 : i]);
+    const bool keep0 = solid && solid[LBRS_IX(i, N, 64)], keep1 = !two || (solid && solid[LBRS_IX(i + 1, N, 64)]);
     const bool vec = (N & 1) == 0 && !keep0 && !keep1;   // every plane starts on 8 bytes
     MarchConst m;
     m.c = pk(c, c);
@@ -156,14 +156,14 @@ __global__ void __launch_bounds__(256) equilibria_2d_kernel(const float* __restr
     P2 u[4], e[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float* p = U + k * N + i;
+        const float* p = U + LBRS_IX(k * N + i, 4 * N, 64);
         u[k] = pk(p[0], two ? p[1] : p[0]);
     }
     const MarchPrim pr = march_prim(u[0], u[1], u[2], u[3], m);
     auto store = [&](int k) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            float* p = f + (q * 4 + k) * N + i;
+            float* p = f + LBRS_IX((q * 4 + k) * N + i, 16 * N, 64);
             if (vec) {
                 *reinterpret_cast<P2*>(p) = e[q];
             } else {
