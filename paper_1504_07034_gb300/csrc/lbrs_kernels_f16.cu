@@ -596,7 +596,6 @@ __global__ void __launch_bounds__(kUThreads, F16 ? 3 : 4) step2d_u2_kernel(const
     }
     if (F16 || !inside) wall_relations(a, j, f);
     const int64_t c = (int64_t)j * a.nx + i;
-#pragma unroll
     float U[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -713,7 +712,7 @@ cudaError_t launch_step2_f32u(const F16StepArgs& s, cudaStream_t st)
     const dim3 grid((unsigned)((s.nx + kUX - 1) / kUX), (unsigned)((s.ny + kUY - 1) / kUY));
     if (s.walls)
         return launch_in_chain(s.chained, step2d_u2_kernel<false, true, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
-    if ((int64_t)grid.x * grid.y <= 152)
+    if ((int64_t)grid.x * grid.y <= kSMs)
         return launch_in_chain(s.chained, step2d_u2_kernel<false, false, false, true>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
     return launch_in_chain(s.chained, step2d_u2_kernel<false, false, false>, grid, kUThreads, st, tile_args(s, false), AdaptPair{});
 }
@@ -752,7 +751,7 @@ cudaError_t launch_set_state_f32u(const void* W, int w_dtype, int kind, void* fs
                                   double gamma, cudaStream_t st)
 {
     int64_t b = (N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     const int g = (int)(b < 1 ? 1 : b);
     if (w_dtype == 0) set_state_f16neq_kernel<double><<<g, 256, 0, st>>>((const double*)W, (float*)fs, nullptr, N, plane, kind, gamma);
     else set_state_f16neq_kernel<float><<<g, 256, 0, st>>>((const float*)W, (float*)fs, nullptr, N, plane, kind, gamma);
@@ -764,7 +763,7 @@ cudaError_t launch_set_state_f16neq(const void* W, int w_dtype, int kind, void* 
 {
     float* scale = (float*)((char*)fs + 40 * N);
     int64_t b = (N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     const int g = (int)(b < 1 ? 1 : b);
     float* U = (float*)fs;
     __half* gq = (__half*)((char*)fs + 16 * N);

@@ -2001,7 +2001,7 @@ cudaError_t launch_adapt_step_f32(const StepArgs<float>& a, void* st, double gam
 cudaError_t launch_adapt_init_bound_f32(const void* fs, int64_t N, double gamma, void* st, cudaStream_t s)
 {
     int64_t b = (N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     adapt_init_bound_kernel<float><<<(unsigned)(b < 1 ? 1 : b), 256, 0, s>>>((const float*)fs, N, gamma, (AdaptState*)st);
     return cudaGetLastError();
 }
@@ -2026,7 +2026,7 @@ cudaError_t launch_adjoint_f32(const AdjArgs<float>& a, cudaStream_t s)
 cudaError_t launch_adj_local_f32(const AdjArgs<float>& a, cudaStream_t s)
 {
     int64_t b = (a.N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     adj_local_kernel<<<(unsigned)(b < 1 ? 1 : b), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -2070,7 +2070,7 @@ bool adj_uform_enabled()
 cudaError_t launch_adj_local_u_f32(const AdjArgs<float>& a, cudaStream_t s)
 {
     int64_t b = (a.N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     adj_local_u_kernel<<<(unsigned)(b < 1 ? 1 : b), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -2096,7 +2096,7 @@ cudaError_t launch_adj_fused2_u_f32(const AdjArgs<float>& a, const float* U2, cu
 cudaError_t launch_vjp_equilibrium_f32(const AdjArgs<float>& a, cudaStream_t s)
 {
     int64_t b = (a.N + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
+    if (b > kSMs * 16) b = kSMs * 16;
     vjp_equilibrium2d_kernel<float><<<(unsigned)(b < 1 ? 1 : b), 256, 0, s>>>(a);
     return cudaGetLastError();
 }

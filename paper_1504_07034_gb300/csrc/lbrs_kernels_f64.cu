@@ -17,12 +17,12 @@ namespace lbrs {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kDiagBlocks = 608;   // 4 x 152 SMs; fixed so the reduction order never changes
+constexpr int kDiagBlocks = 4 * kSMs;   // fixed so the reduction order never changes
 
 int grid_for(int64_t n)
 {
     int64_t b = (n + kThreads - 1) / kThreads;
-    const int64_t cap = 152 * 16;
+    const int64_t cap = kSMs * 16;
     if (b > cap) b = cap;
     return b < 1 ? 1 : (int)b;
 }
@@ -896,7 +896,7 @@ cudaError_t launch_adapt_init_bound_f64(const void* fs, int64_t N, double gamma,
 int tube_f64_steps(int64_t nx)
 {
     for (int h : {48, 32, 24})
-        if (nx <= 152 * (kTubeWin64 - 2 * h)) return h;
+        if (nx <= kSMs * (kTubeWin64 - 2 * h)) return h;
     return 16;
 }
 

@@ -193,7 +193,7 @@ bool fmarch_enabled()
 // 1.92 at 3; 1000 x 1000 at 10 rows 11.6, at 8 in two waves 13.2), 8 where a wave would take more than 12.
 static int64_t fmarch_wave_rows(int nx, int ny)
 {
-    const int64_t slots = 152 * kFMBlocks;
+    const int64_t slots = kSMs * kFMBlocks;
     return ((int64_t)((nx + kFMOwn - 1) / kFMOwn) * ny + slots - 1) / slots;
 }
 

@@ -13,7 +13,7 @@ namespace lbrs {
 
 namespace {
 
-constexpr int kSMs = 152, kWarpsPerSM = 16;   // the march's registers allow 16 one-warp blocks per SM
+constexpr int kWarpsPerSM = 16;   // the march's registers allow 16 one-warp blocks per SM
 
 // Moments of the next step's pull from stored distributions: U = sum_q f*_q(x - c_q).  WALLS: with
 // internal walls (solid cells: the moments of what they hold).

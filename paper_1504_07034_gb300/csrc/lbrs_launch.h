@@ -23,6 +23,8 @@ struct NvtxRange {
 
 namespace lbrs {
 
+constexpr int kSMs = 152;      // of the chip that the library is built for
+
 template <typename T>
 struct StepArgs;
 template <typename T>

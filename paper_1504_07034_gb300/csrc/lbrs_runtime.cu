@@ -273,11 +273,11 @@ StepArgs<T> step_args(const lbrs_ctx* ctx, int from)
     return a;
 }
 
-// Arguments of the reduced-state kernels (FP16 non-equilibrium and moments-only forms).
 // Is s being captured into a graph of the library's own?  Its launches then chain (lbrs_chain.cuh); a
 // caller's capture gets ordinary ones.
 bool own_capture(const lbrs_ctx* ctx, cudaStream_t s) { return ctx->cap_stream && s == ctx->cap_stream; }
 
+// Arguments of the reduced-state kernels (FP16 non-equilibrium and moments-only forms).
 F16StepArgs f16_args(const lbrs_ctx* ctx, int from)
 {
     F16StepArgs a;

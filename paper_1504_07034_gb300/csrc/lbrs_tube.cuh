@@ -194,7 +194,7 @@ __device__ __forceinline__ void tube_step_u(P2 U[C / 2][3], const TubeConst& m, 
 
 // One step of the general collision on the stored populations: L moves to -x, Z rests, R moves to
 // +x.
-template <int Q, int C, bool OM1>
+template <int Q, int C>
 __device__ __forceinline__ void tube_step_f(P2 L[C / 2][3], P2 Z[C / 2][3], P2 R[C / 2][3], const TubeConst& m,
                                             const TubeEnds& w)
 {
@@ -223,9 +223,9 @@ __device__ __forceinline__ void tube_step_f(P2 L[C / 2][3], P2 Z[C / 2][3], P2 R
         tube_feq<Q>(U, m, l, z, r);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            L[j][k] = OM1 ? l[k] : fma2(m.om1, gl[k], mul2(m.om, l[k]));
-            if constexpr (Q == 3) Z[j][k] = OM1 ? z[k] : fma2(m.om1, Z[j][k], mul2(m.om, z[k]));
-            R[j][k] = OM1 ? r[k] : fma2(m.om1, gr[k], mul2(m.om, r[k]));
+            L[j][k] = fma2(m.om1, gl[k], mul2(m.om, l[k]));
+            if constexpr (Q == 3) Z[j][k] = fma2(m.om1, Z[j][k], mul2(m.om, z[k]));
+            R[j][k] = fma2(m.om1, gr[k], mul2(m.om, r[k]));
         }
     }
 }
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(32 * kTubeWarps) tube_kernel(const __grid_cons
         load3(0, L);
         if constexpr (Q == 3) load3(1, Z);
         load3(Q - 1, R);
-        for (int s = 0; s < ns; ++s) tube_step_f<Q, C, false>(L, Z, R, m, w);
+        for (int s = 0; s < ns; ++s) tube_step_f<Q, C>(L, Z, R, m, w);
         if constexpr (Q == 3)
             if (tube_not_finite<C>(Z)) return tube_redo<C>(a, c, first, end, off, len, x0, ns, t0, tlen);
         store3(0, L);
