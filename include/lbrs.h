@@ -506,7 +506,8 @@ typedef struct {
  * cells, of which `halo` on each side are recomputed context and the rest
  * (the tile, >= 32 cells) is advanced by up to `halo` steps per launch.  FP32
  * tubes with halo <= 64 step in registers on windows of the kernel's own; of
- * the tuning they take the halo (default 32). */
+ * the tuning they take the halo (default 32).  D1Q2 tubes do so from 128 cells
+ * in the mean on. */
 typedef struct {
     int32_t block, cells_per_thread, halo, reserved;
 } lbrs_batch_tuning;

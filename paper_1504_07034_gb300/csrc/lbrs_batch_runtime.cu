@@ -167,8 +167,13 @@ bool tuning_ok(const lbrs_batch_tuning& t)
 }
 
 // FP32 tubes with up to kTubeMaxHalo steps a launch run in registers (lbrs_tube.cuh): the tiles
-// follow from the halo alone.
-bool in_registers(const lbrs_batch* B, const lbrs_batch_tuning& t) { return !B->f64 && t.halo <= kTubeMaxHalo; }
+// follow from the halo alone.  Not D1Q2 tubes of fewer than 128 cells in the mean, of which a warp's window
+// would hold little (omega = 1, 200 steps, shared memory and registers, ms: 46875 tubes of 64 cells 3.40, 3.63;
+// 30000 of 100 cells 2.72, 2.92; 187500 of 16 cells 13.1, 14.3; 15000 of 200 cells 1.91, 1.52).
+bool in_registers(const lbrs_batch* B, const lbrs_batch_tuning& t)
+{
+    return !B->f64 && t.halo <= kTubeMaxHalo && (B->q == 3 || B->N >= 128 * B->cfg.batch);
+}
 
 int tile_of(const lbrs_batch_tuning& t) { return t.block * t.cells_per_thread - 2 * t.halo; }
 
@@ -352,7 +357,8 @@ lbrs_status lbrs_batch_create(const lbrs_batch_config* cfg, void* d_workspace, s
     B->f[1] = B->ws + L.f1;
     B->stream = (cudaStream_t)cfg->cuda_stream;
     // FP32: 32 steps a launch (4096 tubes: 52.9 ms; 16 steps 68.3, 48 steps 52.0, 64 steps 54.0)
-    B->tuning = B->f64 ? lbrs_batch_tuning{256, 2, 16, 0} : lbrs_batch_tuning{256, 4, 32, 0};
+    B->tuning = lbrs_batch_tuning{256, 4, 32, 0};
+    if (!in_registers(B, B->tuning)) B->tuning = lbrs_batch_tuning{256, 2, 16, 0};
     // tube tables
     std::vector<int64_t> off(cfg->batch);
     std::vector<int> len(cfg->batch);

@@ -169,3 +169,29 @@ def test_repeated_batch_runs():
         assert torch.equal(a.get_distributions(), c.get_distributions()), (lattice, omega)
         a.close()
         c.close()
+
+
+@pytest.mark.parametrize("lattice, cells, in_registers", [("d1q2", 127, False), ("d1q2", 128, True), ("d1q2", 16, False),
+                                                         ("d1q3", 16, True)])
+def test_batches_of_tiny_tubes(lattice, cells, in_registers):
+    """D1Q2 tubes of few cells step in shared memory (16 steps a launch), others in registers (32), with the same
+    bits as by the other kernel (halo 65 is beyond the register kernel's)."""
+    import torch
+    from paper_1504_07034_gb300.solver import BatchSolver
+    count, steps = 50, np.full(50, 40)
+    x = torch.arange(count * cells, device="cuda").double()
+    W = torch.stack([1.0 + 0.1 * torch.cos(x / 7), 0.1 * torch.sin(x / 5), 1.0 - 0.1 * torch.sin(x / 11)])
+    res = []
+    for tuning in (None, (256, 2, 65)):
+        b = BatchSolver([cells] * count, [4.0] * count, precision="f32", lattice=lattice)
+        if tuning:
+            b.tuning = tuning
+        b.set_state(W)
+        n0 = b.launch_count
+        b.run(steps)
+        launches = b.launch_count - n0
+        res.append(b.get_distributions())
+        if tuning is None:
+            assert launches == (2 if in_registers else 3)
+        b.close()
+    assert torch.equal(res[0], res[1])
