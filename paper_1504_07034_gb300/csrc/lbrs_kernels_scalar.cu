@@ -64,10 +64,16 @@ ScalarPlan scalar_plan(int nx, int ny, const int bc[4])
         p.steps = 512;
         p.min_steps = cells <= 5200 ? 4 : 5;
         if (threads_for(p.wx, p.wy, p.rows) <= 1024) return p;
+        p = ScalarPlan{};
     }
-    p.wx = cells < 1000000 ? 64 : 128;
-    p.wy = cells < 150000 ? 32 : 64;
-    p.rows = cells < 1000000 ? 4 : 8;
+    // Flat grids keep the low windows, whose rows they fill better (40 steps, us, low and high ones: 20000 x 8 89,
+    // 150; 65536 x 12 207, 392; 200000 x 16 563, 935; 65536 x 20 374, 338), and the flattest large ones the two-step
+    // kernel (10 steps, us, windows and that kernel: 200000 x 4 187, 147; 65536 x 4 71, 65; 200000 x 6 153, 157).
+    if (ny < 6 && cells >= 100000) return p;
+    const bool flat = ny <= 16, wide = cells >= 1000000 && !flat;
+    p.wx = wide ? 128 : 64;
+    p.wy = cells < 150000 || flat ? 32 : 64;
+    p.rows = wide ? 8 : 4;
     p.hx = p.hy = p.steps = 8;
     p.tx = p.wx - 16;
     p.ty = p.wy - 16;

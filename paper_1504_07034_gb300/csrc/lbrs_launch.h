@@ -187,7 +187,7 @@ cudaError_t launch_wall_codes(const StepArgs<float>& a, uint8_t* codes, cudaStre
 struct ScalarPlan {
     int wx, wy, hx, hy, tx, ty;   // window, cells beyond the tile, tile
     int rows;                     // rows a thread owns
-    int steps;                    // steps per launch at most
+    int steps;                    // steps per launch at most (0: no windows)
     int min_steps;                // calls of fewer steps keep the two-step kernel,
     int tail;                     // as does a last launch of at most so many
 };

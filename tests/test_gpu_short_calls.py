@@ -195,3 +195,11 @@ def test_batches_of_tiny_tubes(lattice, cells, in_registers):
             assert launches == (2 if in_registers else 3)
         b.close()
     assert torch.equal(res[0], res[1])
+
+
+def test_flat_scalar_grids(tmp_path):
+    """Grids of few rows fill the windows' rows badly."""
+    sizes = [(20000, 8, (10, 40)), (20000, 12, (10,)), (65536, 4, (10, 40)), (65536, 8, (10, 40)), (65536, 16, (10, 40)),
+             (65536, 20, (10,)), (200000, 2, (10,)), (200000, 6, (10, 40)), (200000, 16, (10,))]
+    _compare(tmp_path, [{"kind": "scalar", "nx": nx, "ny": ny, "n": n} for nx, ny, ns in sizes for n in ns],
+             {"LBRS_F32S_WINDOW": "0"})
