@@ -466,10 +466,16 @@ cudaError_t launch_u_steps(const lbrs_ctx* ctx, const char* src, char* dst, int 
 // storing step beside (step_march), worth it later as the traffic of the three grows beside the pairs'
 // (us on the moments and by storing steps, 1800 x 600 6 steps 128 and 122; 2400 x 800 6, 8 steps 210 and 167,
 // 245 and 222; 2048 x 1024 10 steps 304 and 290; 4096 x 1024 10, 12 steps 571 and 516, 647 and 618).
-int64_t march_min(const lbrs_ctx* ctx, int64_t n)
+// Small grids whose sides no tensor copy takes step two a launch outside a graph as fast as the moments do
+// (130^2, 257 x 64: 8, 10, 16 steps 33, 40, 58 us on the moments and 28, 34, 52 by storing pairs), so that
+// entry and exit pay from the first graph on; recording steps have none (201^2, clamped sides: 8, 10, 16, 24 steps
+// 34, 41, 59, 84 us and 30, 37, 58, 85; 257^2 periodic: 8, 10, 16 steps 35, 40, 58 and 36, 44, 68).
+int64_t march_min(const lbrs_ctx* ctx, int64_t n, bool record = false)
 {
     if (ctx->solid && n % 2 == 0 && ctx->N >= 1000000)
         return ctx->N < 1500000 ? 8 : (ctx->N < 2000000 ? 10 : (ctx->N < 4000000 ? 12 : 14));
+    if (!ctx->solid && ctx->N < 60000 && !step3_tiles(ctx))
+        return ctx->N >= 30000 ? 16 : (record ? INT64_MAX : 2 * kGraphSteps + 1);
     return ctx->N < 400000 ? 8 : 6;
 }
 
@@ -799,7 +805,7 @@ cudaError_t launch_equilibria_from(lbrs_ctx* ctx, const char* U, const uint8_t* 
 lbrs_status record_steps(lbrs_ctx* ctx, int64_t n, char* U_hist)
 {
     const size_t stride = (size_t)ctx->K * ctx->N * elem_bytes(ctx);
-    if (march(ctx) && n >= march_min(ctx, n)) {
+    if (march(ctx) && n >= march_min(ctx, n, true)) {
         LBRS_CUDA(ctx, launch_pull_into(ctx, ctx->f[ctx->cur], U_hist));
         lbrs_status st = record_march(ctx, U_hist, n - 1, U_hist + stride);
         if (st != LBRS_OK) return st;
