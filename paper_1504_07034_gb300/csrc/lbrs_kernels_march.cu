@@ -261,6 +261,7 @@ static int march_mode()
 }
 
 bool march_enabled() { return march_mode() != 0; }
+bool march_always() { return march_mode() >= 2; }
 
 // The tile kernel's two-step launch (step2d_u2_kernel, 32 x 16 tiles, four blocks per SM) starts
 // faster than a march and wins on small grids: about 2.7 us and 1.05 us per tile of an SM against the
@@ -271,7 +272,7 @@ bool march_enabled() { return march_mode() != 0; }
 // and side sets from 64^2 to 1531 x 973 the choice is at most 4 % slower than the other kernel.)
 bool march_prefers_tiles(int nx, int ny, const int bc[4])
 {
-    if (march_mode() >= 2) return false;
+    if (march_always()) return false;
     MarchArgs a;
     a.nx = nx;
     a.ny = ny;

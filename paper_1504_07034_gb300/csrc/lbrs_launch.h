@@ -166,8 +166,8 @@ struct MarchStep {
     bool chained;              // the next of a captured chain (lbrs_chain.cuh)
 };
 bool march_enabled();
-// The moments-only form's tile kernels (launch_step2_f32u) are faster on this grid; never with
-// LBRS_F32_MARCH=2.
+bool march_always();           // LBRS_F32_MARCH=2: on every grid, also where tiles or storing steps are faster
+// The moments-only form's tile kernels (launch_step2_f32u) are faster on this grid; never if march_always.
 bool march_prefers_tiles(int nx, int ny, const int bc[4]);
 
 void march_ghosts(const GhostSpec& g, double gamma, double c, float out[4][16]);

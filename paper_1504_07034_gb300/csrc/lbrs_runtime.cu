@@ -474,7 +474,7 @@ int64_t march_min(const lbrs_ctx* ctx, int64_t n, bool record = false)
 {
     if (ctx->solid && n % 2 == 0 && ctx->N >= 1000000)
         return ctx->N < 1500000 ? 8 : (ctx->N < 2000000 ? 10 : (ctx->N < 4000000 ? 12 : 14));
-    if (!ctx->solid && ctx->N < 60000 && !step3_tiles(ctx))
+    if (!ctx->solid && ctx->N < 60000 && !step3_tiles(ctx) && !march_always())
         return ctx->N >= 30000 ? 16 : (record ? INT64_MAX : 2 * kGraphSteps + 1);
     return ctx->N < 400000 ? 8 : 6;
 }
