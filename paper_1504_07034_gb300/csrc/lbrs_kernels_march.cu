@@ -245,6 +245,7 @@ cudaError_t launch_k(MarchArgs a, bool chained, cudaStream_t s)
     // pairs of columns move as 8-byte words where every row starts on one: nx even, and (moments recorded into
     // a caller's buffer) the buffers themselves on 8 bytes
     const bool words = (a.nx & 1) || (((uintptr_t)a.src | (uintptr_t)a.dst) & 7);
+    chained = chained && !RECORD;
     if (words) return launch_in_chain(chained, march2d_kernel<K, true, RECORD>, (unsigned)blocks, 32, s, a);
     return launch_in_chain(chained, march2d_kernel<K, false, RECORD>, (unsigned)blocks, 32, s, a);
 }

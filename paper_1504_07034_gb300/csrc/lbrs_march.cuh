@@ -249,12 +249,17 @@ __device__ __forceinline__ P2 march_bottom(P2 S, const MarchArgs& a, const March
 
 // Two columns x[0], x[1] (adjacent on an 8-byte boundary unless ODD) of the row at offset `row` of an
 // array of n values.  The offset is the same for all lanes, which leaves the address arithmetic to
-// the uniform data path.
-template <bool ODD>
+// the uniform data path.  CHAINED: the launch before may still be writing the array (lbrs_chain.cuh).
+template <bool ODD, bool CHAINED>
 __device__ __forceinline__ P2 march_load2(const float* p, int64_t n, int64_t row, const int x[2])
 {
-    if constexpr (ODD) return pk(chain_load(p + LBRS_IX(row + x[0], n, 51)), chain_load(p + LBRS_IX(row + x[1], n, 51)));
-    else return chain_load(reinterpret_cast<const P2*>(p + LBRS_IX(row + x[0], n - 1, 51)));
+    if constexpr (CHAINED) {
+        if constexpr (ODD) return pk(chain_load(p + LBRS_IX(row + x[0], n, 51)), chain_load(p + LBRS_IX(row + x[1], n, 51)));
+        else return chain_load(reinterpret_cast<const P2*>(p + LBRS_IX(row + x[0], n - 1, 51)));
+    } else {
+        if constexpr (ODD) return pk(__ldg(p + LBRS_IX(row + x[0], n, 51)), __ldg(p + LBRS_IX(row + x[1], n, 51)));
+        else return __ldg(reinterpret_cast<const P2*>(p + LBRS_IX(row + x[0], n - 1, 51)));
+    }
 }
 
 template <bool ODD>
@@ -334,7 +339,7 @@ __device__ __forceinline__ void march_rows(const MarchArgs& a, const MarchPlace&
     for (int n = 0; n < 2; ++n) {
         const int64_t row = fetch_row();
 #pragma unroll
-        for (int k = 0; k < 4; ++k) nxt[n][k] = march_load2<ODD>(a.src, 4 * a.N, k * a.N + row, x);
+        for (int k = 0; k < 4; ++k) nxt[n][k] = march_load2<ODD, !RECORD>(a.src, 4 * a.N, k * a.N + row, x);
     }
     auto iteration = [&](auto parity) {
         constexpr int p = decltype(parity)::value;
@@ -343,7 +348,7 @@ __device__ __forceinline__ void march_rows(const MarchArgs& a, const MarchPlace&
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             U[k] = nxt[p][k];
-            nxt[p][k] = march_load2<ODD>(a.src, 4 * a.N, k * a.N + in, x);
+            nxt[p][k] = march_load2<ODD, !RECORD>(a.src, 4 * a.N, k * a.N + in, x);
         }
 #pragma unroll
         for (int s = 0; s < K; ++s) {
@@ -398,7 +403,8 @@ __device__ __forceinline__ void march_rows(const MarchArgs& a, const MarchPlace&
     }
 }
 
-// K steps a launch, one warp a block.  RECORD: every step's moments are stored.
+// K steps a launch, one warp a block.  RECORD: every step's moments are stored; such launches are never links
+// of a chain and read by __ldg (backward pass of 2048^2, 400 steps: 23.7 ms, 24.1 with a chain's loads).
 template <int K, bool ODD, bool RECORD>
 __global__ void __launch_bounds__(32, 16) march2d_kernel(const __grid_constant__ MarchArgs a)
 {

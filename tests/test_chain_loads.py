@@ -57,6 +57,8 @@ def test_chained_kernels_read_behind_the_wait(kernel):
     first = load.search(body)
     assert first and "chain_begin();" in body[:first.start()]
     for b in bodies:
+        if "if constexpr (CHAINED) {" in b:              # the other branch is of launches outside chains
+            b = b[:b.index("} else {")]
         assert "__ldg" not in b
         assert not re.search(rf"\ba\.({names})\s*\[|\*\s*a\.({names})\b", b)
     assert any("chain_load(" in b for b in bodies)
@@ -64,6 +66,16 @@ def test_chained_kernels_read_behind_the_wait(kernel):
     for m in members:
         decl = re.search(rf"[^;{{}}]*\b{m};", struct).group(0)
         assert "__restrict__" not in decl, decl
+
+
+def test_unchained_loads_belong_to_unchained_launches():
+    """march_load2's read-only loads are the recording form's, which is never launched in a chain."""
+    march = _read("lbrs_march.cuh")
+    calls = re.findall(r"march_load2<([^>]*)>\(a\.src", march)
+    assert calls and all(c == "ODD, !RECORD" for c in calls)
+    unit = _read("lbrs_kernels_march.cu")
+    body = _body(unit, r"cudaError_t launch_k\(")
+    assert body.index("chained = chained && !RECORD;") < body.index("launch_in_chain(")
 
 
 def test_chain_load_keeps_its_place():
