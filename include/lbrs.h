@@ -441,7 +441,8 @@ lbrs_status lbrs_rows_import(lbrs_ctx* ctx, int side, void* d_buf, int planes, c
  * contexts, get LBRS_EINVAL. */
 
 /* Enqueue n steps like lbrs_step, also writing each step's moments U^{s+m+1}
- * (the U its collision used) to d_U_hist + m*K*N elements, m = 0..n-1. */
+ * (the U its collision used) to d_U_hist + m*K*N elements, m = 0..n-1; d_U_hist
+ * needs no alignment beyond its elements'. */
 lbrs_status lbrs_step_record(lbrs_ctx* ctx, int64_t n, void* d_U_hist);
 
 /* gbar[q][k] = dL/dU_k for every q (U_k = sum_q f*_{q,k}); d_dLdU is [K][ny][nx] of dtype. */
